@@ -43,6 +43,7 @@ struct Carver {
 
 struct Shape {
   int n, npad, K, S, W, T, NT, nblk;
+  int split;   // warps sharing a tile pair's partner steps
   size_t dcb;  // divide-and-conquer tree scratch (0 unless that builder is selected)
 };
 
@@ -55,6 +56,7 @@ Shape shape_of(int n, const mstar_params& p) {
   s.K = p.k_fix;
   s.S = p.k_fix + 1;
   s.NT = s.npad / s.T;
+  s.split = s.W != 1 ? 1 : (p.pair_split ? p.pair_split : (n <= 512 ? 4 : 1));
   s.nblk = (s.npad + kBlock - 1) / kBlock;
   s.dcb = p.mst_method == 1 ? dc_scratch_bytes(n, p.mst_nsub) : 0;
   return s;
@@ -76,6 +78,7 @@ size_t carve(const Shape& s, void* base, Dev* d, double** stage) {
   t.child_off = c.take<int>(np + 1);
   t.child_idx = c.take<int>(np);
   t.bylev = c.take<int>(np);
+  t.near_words = s.split == 1 ? c.take<unsigned>(np / 32 * np) : nullptr;
   t.X0 = c.take<double>(n3);
   t.V0 = c.take<double>(n3);
   t.A0 = c.take<double>(n3);
@@ -674,7 +677,7 @@ int mstar_init(mstar_ctx** out, int n, const double* m, const double* r, const d
   c->T = s.T;
   c->NT = s.NT;
   c->ntp = s.NT * (s.NT + 1) / 2;
-  c->S = s.W != 1 ? 1 : (p->pair_split ? p->pair_split : (n <= 512 ? 4 : 1));
+  c->S = s.split;
   // how an attempt's divisions are issued: one CTA per division (pair sums included) for small
   // systems, else a stream per division from 1000 bodies, else level by level
   const int ds = p->division_schedule;

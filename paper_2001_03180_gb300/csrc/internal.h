@@ -34,6 +34,7 @@ struct Dev {
   int* child_off;   // [npad + 1] CSR of children
   int* child_idx;   // [npad]
   int* bylev;       // [npad] the bodies in order of tree level, then index (path-sum order)
+  unsigned* near_words;  // npad / 32 rows of npad words: the tree's near pairs (tiled pair loop; else null)
   double* X0;       // edge vectors of the step start (3 planes)
   double* V0;
   double* A0;       // relative accelerations a_v - a_parent(v) at the step start
@@ -159,6 +160,7 @@ constexpr int kDcMaxSub = 1024;              // largest subgraph count the GPU b
 
 // pair.cu: slots [slot_lo, slot_hi) -> sa, Ublk. n_d as in params (0 = all Cartesian).
 cudaError_t launch_forces(mstar_ctx* c, int slot_lo, int slot_hi, int n_d);
+cudaError_t launch_near_words(mstar_ctx* c);  // the near-pair masks of the current tree
 // at context creation: every kernel of an attempt prefers the largest shared-memory share, so that
 // the CTAs of different kernels can share an SM (a hint; nothing fails without it)
 void prefer_shared_pair_kernels();

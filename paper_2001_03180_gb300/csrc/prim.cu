@@ -448,7 +448,9 @@ cudaError_t launch_tree(mstar_ctx* c) {
   k_tree<<<1, 1024, smem, c->stream>>>(c->n, c->npad, c->d.parent, c->d.level, c->d.gp, c->d.child_off,
                                        c->d.child_idx, c->d.bylev);
   MSTAR_LAUNCHED(c);
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_near_words(c);
 }
 
 }  // namespace mstar
