@@ -62,3 +62,18 @@ def test_rebuild_test_rejects_bad_arguments():
         M.mstar_rebuild_test([(m, r, v)], [0], [4], 1, 1, [0])
     with pytest.raises(M.MstarError):
         M.mstar_rebuild_test([(m, r, v)], [0], [0], 5, 1, [3, 2])
+
+
+@pytest.mark.parametrize("copies", [5, 12, 25, 60])
+def test_cluster_sizes_give_the_same_bits(copies):
+    """The more jobs a call has, the smaller the cluster each gets (16 CTAs down to one): the same
+    eight jobs, alone and repeated, give the same bits, and those of the CPU definition."""
+    n = 70
+    m, r, v, _ = W.hernquist(n, 3)
+    jobs = [(c, d) for c in (0, 1) for d in (0, 1, 2, 3)]
+    one = M.mstar_rebuild_test([(m, r, v)] * 8, [j[0] for j in jobs], [j[1] for j in jobs], 21, 10, [0, 7, 21])
+    many = M.mstar_rebuild_test([(m, r, v)] * (8 * copies), [j[0] for j in jobs] * copies, [j[1] for j in jobs] * copies,
+                                21, 10, [0, 7, 21])
+    for key in ("E", "r", "v", "topo_changes", "mean_level"):
+        for k in range(copies):
+            assert np.array_equal(many[key][8 * k:8 * k + 8], one[key]), (key, k)
