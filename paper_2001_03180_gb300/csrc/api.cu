@@ -831,6 +831,7 @@ int mstar_get_mst(mstar_ctx* c, int* root, int* parent, int* level, int* order) 
       CK(launch_tree(c));
       c->mst_valid = true;
     }
+    if (order) CK(launch_bfs_order(c));
   } else if (order) {
     // Prim's kernel records the insertion order; it builds the same tree as the step's
     // MST builder, so the step buffers stay valid.

@@ -8,8 +8,8 @@
 // cheapest outgoing edge, and components merge along those edges. If two different
 // candidates ever compare exactly equal in FP64, the tree could depend on tie-breaking
 // rules, and the caller falls back to the Prim kernel, which applies the paper's rule.
-// The tree is then oriented from Prim's root (the body closest to the centre of mass) by a
-// breadth-first walk, which gives the same parent and level as Prim's indexing.
+// The tree is then oriented from Prim's root (the body closest to the centre of mass), which gives
+// the same parent and level as Prim's indexing.
 //
 // Distances are computed exactly as the CPU definition does: ((dx*dx)+(dy*dy))+(dz*dz)
 // with dx = x_u - x_v, each operation rounded separately.
@@ -269,163 +269,221 @@ __global__ void k_boruvka_init(int n, const double* __restrict__ X, const double
   ccnt[i] = 0;
 }
 
-// Orient the tree from Prim's root: adjacency from the edge list, then a breadth-first
-// walk in one CTA (levels are tree depths, independent of the visiting order). The
-// adjacency, the visited marks and the queue live in shared memory (5n + 1 ints).
+// |x| within [lo, hi] as floats, from the bits of a double (integer operations: a conversion costs
+// an FP64 issue slot). hi is +inf from 2^127 on (and for NaN), lo is 0 below 2^-126.
+__device__ __forceinline__ void abs_bounds(double x, float& lo, float& hi) {
+  const int h = __double2hiint(x) & 0x7fffffff;
+  const int e = (h >> 20) - 1023;
+  const float f = __int_as_float(((e + 127) << 23) | ((h & 0xfffff) << 3));  // truncated: f <= |x| < f (1 + 2^-19)
+  lo = e < -126 ? 0.0f : (e > 126 ? 0x1p126f : f);
+  hi = e < -126 ? 0x1p-125f : (e > 126 ? __int_as_float(0x7f800000) : f * (1.0f + 0x1p-18f));
+}
+
+// Orient the tree from Prim's root (the body closest to the origin, lowest index on ties): parent
+// and level of every vertex from the edge list, in one CTA.
+//
+// Euler tour and list ranking, because a walk level by level is a chain as long as the tree is
+// deep (59 levels at N = 2050, 150 at N = 10002: 57 and 220 us in one warp, which measured faster
+// than block barriers between levels). Edge e gives the arcs 2e (eu -> ev) and 2e + 1 (ev -> eu);
+// the arc after u -> v in the tour is the one after v -> u in v's circular adjacency list. Up to
+// blockDim arcs are splitters: each thread walks from its splitter to the next one (about 20 arcs
+// at N = 10002, in shared memory), the splitters are ranked by pointer doubling, and a second walk
+// gives every arc its rank. An arc that precedes its twin leads away from the root, and the
+// running sum of +1 (away) and -1 (back) along the tour is the level it reaches. Parent and level
+// do not depend on the order of the adjacency lists, which the atomic fill leaves open.
+// 20 n bytes of shared memory hold the arcs as 16-bit numbers (2 (n - 1) < 2^16).
+// N = 601, 2050, 5003, 10002: 28, 57, 122 and 220 us before, 11, 18, 30 and 51 us now.
+constexpr int kNoSplitter = 0xffff;
+static_assert(2 * MSTAR_MAX_N < kNoSplitter, "arcs and splitters must fit 16 bits");
+
 __global__ void __launch_bounds__(1024, 1)
 k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, const double* __restrict__ Z,
-         const int* __restrict__ eu, const int* __restrict__ ev, int* __restrict__ adj_off, int* __restrict__ adj,
-         int* __restrict__ parent, int* __restrict__ level, int* __restrict__ root_out, int* __restrict__ queue) {
+         const int* __restrict__ eu, const int* __restrict__ ev, int* __restrict__ parent, int* __restrict__ level,
+         int* __restrict__ root_out) {
   extern __shared__ int smi[];
-  int* s_off = smi;           // n + 1
-  int* s_adj = s_off + n + 1; // 2 (n - 1)
-  int* s_a = s_adj + 2 * n;   // n: degrees, then the parents
-  int* s_q = s_a + n;         // n: fill counters, then the queue
+  typedef unsigned short u16;
+  const int na = 2 * (n - 1);
+  int* off = smi;                                    // n: end of each vertex's list (after the fill)
+  u16* src = reinterpret_cast<u16*>(off + n);        // 2 n: source vertex of each arc
+  u16* adj = src + 2 * n;                            // 2 n: arcs by source; then the ranks
+  u16* pos = adj + 2 * n;                            // 2 n: place of each arc in adj; then its splitter; then the arc at each rank
+  u16* succ = pos + 2 * n;                           // 2 n
   __shared__ unsigned long long rk[32];
-  __shared__ int ri[32];
-  __shared__ int part[1024];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int v = tid; v < n; v += nt) {
-    s_a[v] = 0;
-    s_q[v] = 0;
+  __shared__ int ri[32], part[32], s_root;
+  __shared__ float s_hi;
+  __shared__ int s_len[2][1024], s_nxt[2][1024];
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  for (int v = tid; v < n; v += nt) off[v] = 0;
+  // root: float bounds of |r|^2 first, FP64 for the bodies whose lower bound does not exceed the
+  // least upper bound (5 FP64 instructions per body on one SM would take 12 us at N = 10002)
+  float uhi = __int_as_float(0x7f800000);
+  for (int w = tid; w < n; w += nt) {
+    float lx, hx, ly, hy, lz, hz;
+    abs_bounds(X[w], lx, hx);
+    abs_bounds(Y[w], ly, hy);
+    abs_bounds(Z[w], lz, hz);
+    uhi = fminf(uhi, (hx * hx + hy * hy + hz * hz) * (1.0f + 0x1p-20f) + 0x1p-126f);
   }
-  // root: closest to the origin (COM frame), lowest index on ties
+  uhi = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(uhi)));
+  if (lane == 0) rk[warp] = __float_as_uint(uhi);
+  __syncthreads();
+  if (warp == 0) {
+    const unsigned u = __reduce_min_sync(0xffffffffu, lane < nw ? (unsigned)rk[lane] : 0x7f800000u);
+    if (lane == 0) s_hi = __uint_as_float(u);
+  }
+  // (endpoints outside [0, n) cannot come from the tree builders; they are made 0 so that no
+  // shared-memory index leaves its array)
+  for (int e = tid; e < n - 1; e += nt) {
+    int a = eu[e], b = ev[e];
+    if ((unsigned)a >= (unsigned)n || (unsigned)b >= (unsigned)n) a = b = 0;
+    src[2 * e] = (u16)a;
+    src[2 * e + 1] = (u16)b;
+    atomicAdd(&off[a], 1);
+    atomicAdd(&off[b], 1);
+  }
+  __syncthreads();
+  uhi = s_hi;
   unsigned long long bk = ~0ull;
   int bi = INT_MAX;
   for (int w = tid; w < n; w += nt) {
-    const double x = X[w], y = Y[w], z = Z[w];
-    const unsigned long long k =
-        key_bits(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
-    if (k < bk || (k == bk && w < bi)) {
-      bk = k;
-      bi = w;
+    float lx, hx, ly, hy, lz, hz;
+    abs_bounds(X[w], lx, hx);
+    abs_bounds(Y[w], ly, hy);
+    abs_bounds(Z[w], lz, hz);
+    if ((lx * lx + ly * ly + lz * lz) * (1.0f - 0x1p-20f) <= uhi) {
+      const double x = X[w], y = Y[w], z = Z[w];
+      const unsigned long long k =
+          key_bits(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
+      if (k < bk || (k == bk && w < bi)) {
+        bk = k;
+        bi = w;
+      }
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long k2 = __shfl_down_sync(0xffffffffu, bk, o);
-    const int i2 = __shfl_down_sync(0xffffffffu, bi, o);
+    const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, bk, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
     if (k2 < bk || (k2 == bk && i2 < bi)) {
       bk = k2;
       bi = i2;
     }
   }
-  if ((tid & 31) == 0) {
-    rk[tid >> 5] = bk;
-    ri[tid >> 5] = bi;
+  if (lane == 0) {
+    rk[warp] = bk;
+    ri[warp] = bi;
   }
   __syncthreads();
   if (tid == 0) {
-    for (int w = 1; w < (nt >> 5); ++w)
+    for (int w = 1; w < nw; ++w)
       if (rk[w] < rk[0] || (rk[w] == rk[0] && ri[w] < ri[0])) {
         rk[0] = rk[w];
         ri[0] = ri[w];
       }
+    s_root = min(ri[0], n - 1);
+    root_out[0] = s_root;
   }
-  // (endpoints outside [0, n) cannot come from the tree builders; they are skipped so that
-  // no shared-memory index leaves its array)
-  for (int e = tid; e < n - 1; e += nt) {
-    const int a = eu[e], b = ev[e];
-    if ((unsigned)a < (unsigned)n && (unsigned)b < (unsigned)n) {
-      atomicAdd(&s_a[a], 1);
-      atomicAdd(&s_a[b], 1);
-    }
-  }
-  __syncthreads();
-  const int root = ri[0];
   // exclusive scan of the degrees: contiguous chunks per thread, then the chunk sums
   const int chunk = (n + nt - 1) / nt;
-  const int b0 = tid * chunk, b1 = min(n, b0 + chunk);
-  int sum = 0;
-  for (int v = b0; v < b1; ++v) sum += s_a[v];
+  const int b0 = min(n, tid * chunk), b1 = min(n, b0 + chunk);
   {
-    int total;
+    int sum = 0, total;
+    for (int v = b0; v < b1; ++v) sum += off[v];
     sum = block_exclusive_scan(sum, part, &total);
-    if (tid == 0) s_off[n] = total;
-  }
-  for (int v = b0; v < b1; ++v) {
-    s_off[v] = sum;
-    sum += s_a[v];
-  }
-  __syncthreads();
-  for (int e = tid; e < n - 1; e += nt) {
-    const int a = eu[e], b = ev[e];
-    if ((unsigned)a < (unsigned)n && (unsigned)b < (unsigned)n) {
-      s_adj[s_off[a] + atomicAdd(&s_q[a], 1)] = b;
-      s_adj[s_off[b] + atomicAdd(&s_q[b], 1)] = a;
+    for (int v = b0; v < b1; ++v) {
+      const int d = off[v];
+      off[v] = sum;
+      sum += d;
     }
   }
   __syncthreads();
-  for (int v = tid; v < n; v += nt) s_a[v] = -2;  // not yet reached
+  for (int a = tid; a < na; a += nt) {
+    const int p = atomicAdd(&off[src[a]], 1);
+    adj[p] = (u16)a;
+    pos[a] = (u16)p;
+  }
   __syncthreads();
+  const int root = s_root;
+  const int head = adj[root > 0 ? off[root - 1] : 0];
+  for (int a = tid; a < na; a += nt) {  // the arc after a: the one after its twin around v
+    const int t = a ^ 1, v = src[t], q = pos[t] + 1;
+    succ[a] = adj[q < off[v] ? q : (v > 0 ? off[v - 1] : 0)];
+  }
+  __syncthreads();
+  // splitters: the head, and arcs at equal distances by number
+  const int ns = min(nt, na);
+  for (int a = tid; a < na; a += nt) pos[a] = (u16)kNoSplitter;
+  __syncthreads();
+  int mine = -1;
+  if (tid < ns) mine = tid == 0 ? head : (int)((long long)tid * na / ns);
+  if (tid > 0 && mine == head) mine = -1;
+  if (mine >= 0) pos[mine] = (u16)tid;
+  __syncthreads();
+  int len = 0, nxt = 0;
+  if (mine >= 0) {
+    int a = mine;
+    do {
+      a = succ[a];
+      ++len;
+    } while (pos[a] == kNoSplitter && len < na);
+    nxt = pos[a] == kNoSplitter ? 0 : pos[a];
+  }
+  // arcs from each splitter to the end of the tour, by pointer doubling (the segment that returns
+  // to the head is the last one)
+  s_len[0][tid] = len;
+  s_nxt[0][tid] = mine >= 0 ? nxt : 0;  // 0: the end
+  __syncthreads();
+  int h = 0;
+  for (int d = 1; d < ns; d <<= 1, h ^= 1) {
+    const int q = s_nxt[h][tid];
+    s_len[h ^ 1][tid] = s_len[h][tid] + (q ? s_len[h][q] : 0);
+    s_nxt[h ^ 1][tid] = q ? s_nxt[h][q] : 0;
+    __syncthreads();
+  }
+  if (mine >= 0) {
+    int k = na - s_len[h][tid], a = mine;  // rank of the splitter
+    for (int j = 0; j < len; ++j, ++k) {
+      adj[a] = (u16)min(max(k, 0), na - 1);
+      a = succ[a];
+    }
+  }
+  __syncthreads();
+  for (int a = tid; a < na; a += nt) pos[adj[a]] = (u16)a;
+  __syncthreads();
+  const int ca = (na + nt - 1) / nt;
+  const int r0 = min(na, tid * ca), r1 = min(na, r0 + ca);
+  int depth = 0, total;
+  for (int k = r0; k < r1; ++k) {
+    const int a = min((int)pos[k], na - 1);
+    depth += adj[a] < adj[a ^ 1] ? 1 : -1;
+  }
+  depth = block_exclusive_scan(depth, part, &total);
+  for (int k = r0; k < r1; ++k) {
+    const int a = min((int)pos[k], na - 1);
+    const bool away = adj[a] < adj[a ^ 1];
+    depth += away ? 1 : -1;
+    if (away) {
+      parent[src[a ^ 1]] = src[a];
+      level[src[a ^ 1]] = depth;
+    }
+  }
   if (tid == 0) {
-    s_a[root] = -1;
-    s_q[0] = root;
-    root_out[0] = root;
+    parent[root] = -1;
+    level[root] = 0;
   }
-  __syncthreads();
-  // Level by level in warp 0: [h, t) is the current level, taken 32 vertices at a time, one per
-  // lane. Each lane walks its vertex's neighbours; in every round the lanes that found an
-  // unvisited neighbour append it at their rank among them (ballot), so the queue order is
-  // fixed given the adjacency lists and no block barrier is needed between levels (a level holds ~35 vertices on average
-  // at N = 2050, where 59 levels with block barriers cost about 1 us each). In a tree a vertex
-  // is reached from its parent only, so no vertex is appended twice. (Parent and level do not
-  // depend on the order of the adjacency lists, which the atomic fill above leaves open.)
-  if (tid < 32) {
-    const int lane = tid;
-    const unsigned lt = (1u << lane) - 1u;
-    int h = 0, t = 1, depth = 0;
-    while (h < t) {
-      int tail = t;
-      for (int base = h; base < t; base += 32) {
-        const int q = base + lane;
-        const int u = q < t ? s_q[q] : -1;
-        if (u >= 0) level[u] = depth;
-        int a = u >= 0 ? s_off[u] : 0;
-        const int aend = u >= 0 ? s_off[u + 1] : 0;
-        while (__any_sync(0xffffffffu, a < aend)) {
-          int w = -1;
-          if (a < aend) {
-            w = s_adj[a];
-            ++a;
-            if (s_a[w] != -2) w = -1;
-          }
-          const unsigned found = __ballot_sync(0xffffffffu, w >= 0);
-          if (w >= 0) {
-            s_a[w] = u;
-            const int slot = tail + __popc(found & lt);
-            if (slot < n) s_q[slot] = w;
-          }
-          tail += __popc(found);
-          __syncwarp();  // this round's marks and appends are seen by every lane in the next
-        }
-        __syncwarp();
-      }
-      h = t;
-      t = min(tail, n);
-      ++depth;
-    }
-  }
-  __syncthreads();
-  for (int v = tid; v < n; v += nt) {
-    parent[v] = s_a[v];
-    queue[v] = s_q[v];
-  }
-  for (int v = tid; v <= n; v += nt) adj_off[v] = s_off[v];
-  for (int a = tid; a < 2 * (n - 1); a += nt) adj[a] = s_adj[a];
 }
 
 }  // namespace
 
 // Orientation of an undirected spanning tree (edges eu[e]-ev[e], e < n-1) from Prim's root
-// into d.parent, d.level, d.root; `queue` receives the breadth-first order.
-cudaError_t launch_orient(mstar_ctx* c, const int* eu, const int* ev, int* adj_off, int* adj, int* queue) {
+// into d.parent, d.level, d.root.
+cudaError_t launch_orient(mstar_ctx* c, const int* eu, const int* ev) {
   const int n = c->n;
   const double* X = c->d.r;
-  const size_t smem = sizeof(int) * (5 * (size_t)n + 1);
+  const size_t smem = 20 * (size_t)n;
   cudaError_t e = cudaFuncSetAttribute(k_orient, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_orient<<<1, 1024, smem, c->stream>>>(n, X, X + c->npad, X + 2 * (size_t)c->npad, eu, ev, adj_off, adj,
-                                         c->d.parent, c->d.level, c->d.root, queue);
+  k_orient<<<1, 1024, smem, c->stream>>>(n, X, X + c->npad, X + 2 * (size_t)c->npad, eu, ev, c->d.parent,
+                                         c->d.level, c->d.root);
   MSTAR_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -462,9 +520,6 @@ cudaError_t launch_mst_boruvka(mstar_ctx* c, bool* tied) {
   int* nxt = reinterpret_cast<int*>(take(sizeof(int) * npad));
   int* eu = reinterpret_cast<int*>(take(sizeof(int) * npad));
   int* ev = reinterpret_cast<int*>(take(sizeof(int) * npad));
-  int* adj_off = reinterpret_cast<int*>(take(sizeof(int) * (npad + 1)));
-  int* adj = reinterpret_cast<int*>(take(sizeof(int) * 2 * npad));
-  int* queue = reinterpret_cast<int*>(take(sizeof(int) * npad));
   unsigned long long* partD = reinterpret_cast<unsigned long long*>(take(8 * (size_t)npad * nparts));
   int* partJ = reinterpret_cast<int*>(take(sizeof(int) * (size_t)npad * nparts));
   int* flags = reinterpret_cast<int*>(take(sizeof(int) * 4));  // [0] tie, [1] edge count, [2] gate, [3] rounds run
@@ -516,7 +571,7 @@ cudaError_t launch_mst_boruvka(mstar_ctx* c, bool* tied) {
     *tied = true;
     return cudaSuccess;
   }
-  return launch_orient(c, eu, ev, adj_off, adj, queue);
+  return launch_orient(c, eu, ev);
 }
 
 }  // namespace mstar

@@ -67,7 +67,6 @@ struct DcLayout {
   int* kp;                       // Prim parent candidates by sorted position
   DcEdge* W;                     // mc x mc meta weights (a < b entries)
   int *eu, *ev;                  // the n - 1 tree edges
-  int *adj_off, *adj, *queue;    // orientation
   size_t bytes;
 };
 
@@ -99,9 +98,6 @@ DcLayout dc_layout(int n, int nsub, char* base) {
   L.W = reinterpret_cast<DcEdge*>(take(sizeof(DcEdge) * (size_t)L.mc * L.mc));
   L.eu = reinterpret_cast<int*>(take(sizeof(int) * (size_t)n));
   L.ev = reinterpret_cast<int*>(take(sizeof(int) * (size_t)n));
-  L.adj_off = reinterpret_cast<int*>(take(sizeof(int) * (size_t)(n + 1)));
-  L.adj = reinterpret_cast<int*>(take(sizeof(int) * 2 * (size_t)n));
-  L.queue = reinterpret_cast<int*>(take(sizeof(int) * (size_t)n));
   L.bytes = (off + 255) & ~size_t(255);
   return L;
 }
@@ -544,6 +540,34 @@ k_dc_meta_prim(int n, const int* __restrict__ ncell, int mc, const DcEdge* __res
   }
 }
 
+// The breadth-first walk of the tree in one warp: the queue is the order. A level's vertices are
+// taken 32 at a time, one per lane; every lane appends its children (ascending) after those of the
+// lanes before it.
+__global__ void __launch_bounds__(32)
+k_bfs_order(int n, const int* __restrict__ root, const int* __restrict__ child_off, const int* __restrict__ child_idx,
+            int* order) {
+  const int lane = threadIdx.x;
+  if (lane == 0) order[0] = root[0];
+  __syncwarp();
+  int tail = 1;
+  for (int h = 0; h < tail && h < n;) {
+    const int t = min(tail, h + 32);  // vertices appended before this pass, in queue order
+    const int v = h + lane < t ? order[h + lane] : -1;
+    const int c0 = v >= 0 ? child_off[v] : 0, cnt = v >= 0 ? child_off[v + 1] - c0 : 0;
+    int incl = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int at = tail + incl - cnt;
+    for (int k = 0; k < cnt; ++k)
+      if (at + k < n) order[at + k] = child_idx[c0 + k];
+    tail += __shfl_sync(0xffffffffu, incl, 31);
+    h = t;
+    __syncwarp();  // this pass's appends are read by the next
+  }
+}
+
 }  // namespace
 
 size_t dc_scratch_bytes(int n, int nsub) { return dc_layout(n, nsub, nullptr).bytes; }
@@ -578,8 +602,15 @@ cudaError_t launch_mst_dc(mstar_ctx* c) {
   k_dc_meta_prim<<<1, 32, 0, s>>>(n, L.ncell, L.mc, L.W, L.eu, L.ev);
   c->launches += 7;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_orient(c, L.eu, L.ev, L.adj_off, L.adj, L.queue)) != cudaSuccess) return e;
-  return cudaMemcpyAsync(c->d.order, L.queue, sizeof(int) * n, cudaMemcpyDeviceToDevice, s);
+  return launch_orient(c, L.eu, L.ev);
+}
+
+// d.order of a divide-and-conquer tree, from the children lists of launch_tree; only a caller that
+// asks for the order (mstar_get_mst) needs it.
+cudaError_t launch_bfs_order(mstar_ctx* c) {
+  k_bfs_order<<<1, 32, 0, c->stream>>>(c->n, c->d.root, c->d.child_off, c->d.child_idx, c->d.order);
+  MSTAR_LAUNCHED(c);
+  return cudaGetLastError();
 }
 
 }  // namespace mstar

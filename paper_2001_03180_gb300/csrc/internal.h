@@ -151,8 +151,9 @@ cudaError_t launch_tree(mstar_ctx* c);      // grandparents and children CSR
 // boruvka.cu: exact MST by Boruvka rounds; *tied = true asks for the Prim kernel instead
 cudaError_t launch_mst_boruvka(mstar_ctx* c, bool* tied);
 constexpr int kBoruvkaMinN = 512;           // below this Prim in one CTA is as fast
-// BFS orientation of an undirected spanning tree from Prim's root (boruvka.cu)
-cudaError_t launch_orient(mstar_ctx* c, const int* eu, const int* ev, int* adj_off, int* adj, int* queue);
+// orientation of an undirected spanning tree from Prim's root (boruvka.cu)
+cudaError_t launch_orient(mstar_ctx* c, const int* eu, const int* ev);
+cudaError_t launch_bfs_order(mstar_ctx* c);  // breadth-first order of the current tree into d.order (dcmst.cu)
 // dcmst.cu: divide-and-conquer spanning tree of d.r (Sec. 3.3) into parent/level/root/order
 cudaError_t launch_mst_dc(mstar_ctx* c);
 size_t dc_scratch_bytes(int n, int nsub);    // device scratch the builder needs

@@ -785,14 +785,14 @@ void prefer_shared_pair_kernels() {
 }
 
 // Bit s & 31 of word (s >> 5, p): bodies p and s are near (at most n_d tree edges apart), for the
-// tiled pair loop's masks. One thread per body walks its own near partners (its column of words,
-// so no two threads write one word); the words were cleared.
+// tiled pair loop's masks. One thread per body walks its own near partners; the words were cleared.
+// (atomicOr, although no two threads meet in a word: without a result to wait for, 10 -> 6 us.)
 __global__ void __launch_bounds__(kBlock)
 k_near_words(int n, int npad, int n_d, const int* __restrict__ parent, const int* __restrict__ gp,
              const int* __restrict__ child_off, const int* __restrict__ child_idx, unsigned* __restrict__ words) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  auto put = [&](int q) { words[(size_t)(q >> 5) * npad + p] |= 1u << (q & 31); };
+  auto put = [&](int q) { atomicOr(&words[(size_t)(q >> 5) * npad + p], 1u << (q & 31)); };
   const int pp = parent[p];
   if (pp >= 0) put(pp);
   const int c0 = child_off[p], c1 = child_off[p + 1];

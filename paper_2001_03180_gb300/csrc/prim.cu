@@ -305,6 +305,74 @@ k_prim(int n, int npad, const double* __restrict__ r, int* __restrict__ parent_o
   }
 }
 
+// The same lists for larger trees, by counting: the place of body v in (level, index) order, its
+// place among the children lists (the order of (parent, index)) and the start of its own list are
+// the numbers of bodies whose key is smaller, found by comparing all pairs over the whole GPU (each
+// CTA 128 bodies against one part of the others), where one CTA's sort and insertion lists took
+// 19, 44, 62 and 120 us at N = 601, 2050, 5003 and 10002 (5, 8, 15 and 39 now). Keys: level 2^14 + index, parent 2^14 + index
+// (the root, which is no child, last); n <= 2^14.
+constexpr int kTreeCountMinN = 512;  // below, one CTA (k_tree) is as fast as two launches
+constexpr int kTreeParts = 8;
+
+__global__ void __launch_bounds__(128)
+k_tree_count(int n, int npad, const int* __restrict__ parent, const int* __restrict__ level, int* __restrict__ cnt) {
+  __shared__ uint2 s[128];
+  const int v = blockIdx.x * 128 + threadIdx.x, q = blockIdx.y;
+  const int per = (n + kTreeParts - 1) / kTreeParts;
+  const int lo = q * per, hi = min(n, lo + per);
+  auto keys = [&](int u) {
+    const int p = parent[u];
+    return make_uint2(((unsigned)level[u] << 14) | (unsigned)u, p >= 0 ? ((unsigned)p << 14) | (unsigned)u : ~0u);
+  };
+  const uint2 kv = v < n ? keys(v) : make_uint2(0u, 0u);
+  const unsigned own = (unsigned)v << 14;
+  int a = 0, b = 0, c = 0;
+  for (int t = lo; t < hi; t += 128) {
+    __syncthreads();
+    s[threadIdx.x] = t + (int)threadIdx.x < hi ? keys(t + threadIdx.x) : make_uint2(~0u, ~0u);
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < 128; ++k) {
+      const uint2 ku = s[k];
+      a += ku.x < kv.x;
+      b += ku.y < kv.y;
+      c += ku.y < own;
+    }
+  }
+  if (v < n) {
+    int* o = cnt + (size_t)q * 3 * npad + v;
+    o[0] = a;
+    o[npad] = b;
+    o[2 * (size_t)npad] = c;
+  }
+}
+
+__global__ void __launch_bounds__(kBlock)
+k_tree_place(int n, int npad, const int* __restrict__ parent, const int* __restrict__ cnt, int* __restrict__ gp,
+             int* __restrict__ child_off, int* __restrict__ child_idx, int* __restrict__ bylev) {
+  const int v = blockIdx.x * kBlock + threadIdx.x;
+  if (v >= npad) return;
+  if (v >= n) {
+    gp[v] = -3;
+    bylev[v] = v;
+    return;
+  }
+  int a = 0, b = 0, c = 0;
+#pragma unroll
+  for (int q = 0; q < kTreeParts; ++q) {
+    const int* o = cnt + (size_t)q * 3 * npad + v;
+    a += o[0];
+    b += o[npad];
+    c += o[2 * (size_t)npad];
+  }
+  const int p = parent[v];
+  gp[v] = p >= 0 ? parent[p] : -1;
+  bylev[a] = v;
+  if (p >= 0) child_idx[b] = v;
+  child_off[v] = c;
+  if (v == 0) child_off[n] = n - 1;
+}
+
 // Grandparents, the children lists (CSR, each list in ascending index) and the bodies in
 // order of (level, index) of the tree. The last is a bitonic sort of the keys level * 2^14
 // + index (n <= 2^14) in shared memory.
@@ -442,6 +510,20 @@ cudaError_t launch_prim(mstar_ctx* c) {
 }
 
 cudaError_t launch_tree(mstar_ctx* c) {
+  if (c->n >= kTreeCountMinN) {
+    // the counts go into the pair partials (3 kTreeParts npad ints; a context of this size has more),
+    // free while the tree is being built
+    int* cnt = reinterpret_cast<int*>(c->d.P);
+    k_tree_count<<<dim3((c->n + 127) / 128, kTreeParts), 128, 0, c->stream>>>(c->n, c->npad, c->d.parent, c->d.level,
+                                                                              cnt);
+    k_tree_place<<<(c->npad + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(c->n, c->npad, c->d.parent, cnt, c->d.gp,
+                                                                            c->d.child_off, c->d.child_idx,
+                                                                            c->d.bylev);
+    c->launches += 2;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_near_words(c);
+  }
   size_t smem = (size_t)c->n * 2 * sizeof(int);
   cudaError_t e = cudaFuncSetAttribute(k_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
