@@ -18,6 +18,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "nearest.cuh"
 
 namespace mstar {
 namespace {
@@ -29,37 +30,13 @@ __device__ __forceinline__ double d2_exact(const double* X, const double* Y, con
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-// Float bounds of the FP64 squared distance ((dx*dx)+(dy*dy))+(dz*dz) of two vertices from
-// their float copies: each coordinate difference errs by at most (|x_i| + |x_j|) 2^-24 + |dx|
-// 2^-24, and e = e_i + e_j holds (max|coordinate_i| + max|coordinate_j|) 2^-23 + 2e-37.
-// (1 -/+ 2^-20) covers the relative rounding of the float sums of squares and the FP64
-// distance's own (< 2^-50); 2^-144 the absolute rounding (<= 2^-150 per operation) of squares
-// and sums below 2^-126. Overflowing squares make hi infinite, which bounds nothing away.
-__device__ __forceinline__ float d2_lower(float dx, float dy, float dz, float e) {
-  const float lx = fmaxf(fmaf(dx, -0x1p-22f, dx) - e, 0.0f);
-  const float ly = fmaxf(fmaf(dy, -0x1p-22f, dy) - e, 0.0f);
-  const float lz = fmaxf(fmaf(dz, -0x1p-22f, dz) - e, 0.0f);
-  return fmaxf(((lx * lx + ly * ly) + lz * lz) * (1.0f - 0x1p-20f) - 0x1p-144f, 0.0f);
-}
-__device__ __forceinline__ float d2_upper(float dx, float dy, float dz, float e) {
-  const float hx = fmaf(dx, 0x1p-22f, dx) + e, hy = fmaf(dy, 0x1p-22f, dy) + e, hz = fmaf(dz, 0x1p-22f, dz) + e;
-  return ((hx * hx + hy * hy) + hz * hz) * (1.0f + 0x1p-20f) + 0x1p-144f;
-}
-
-constexpr int kNfnList = 4;  // candidates a thread lists for exact evaluation
-
 // Nearest foreign neighbour (smallest exact squared distance to a vertex of another
 // component) of every vertex whose cached neighbour is missing or has become internal;
 // CTA (tile, part) scans the part-th slice of the candidates. Writes per (vertex, part)
 // the exact distance bits and the neighbour; exact equal distances to two different
-// candidates at the minimum set *tie.
-//
-// Three steps, so that the FP64 distances (and their divergent, long-latency code) run only
-// for the few candidates that can be the nearest: the least float upper bound over the
-// foreign candidates; the candidates whose float lower bound does not exceed it, listed in
-// index order (a candidate above it is strictly farther than the nearest); their exact
-// distances. A vertex with more than kNfnList listed candidates scans the part again, taking
-// the exact distance of every candidate whose lower bound does not exceed the bound.
+// candidates at the minimum set *tie. One float pass and one exact distance per vertex
+// (NearestScan), where two float passes with upper and lower bounds of 22 instructions a candidate
+// each took 17, 17, 52 and 193 us per round at N = 601, 2050, 5003 and 10002; 6, 7, 20 and 70 now.
 __global__ void __launch_bounds__(kBT)
 k_nfn(int n, int npad, int nparts, const double* __restrict__ X, const double* __restrict__ Y,
       const double* __restrict__ Z, const float* __restrict__ f4, const int* __restrict__ comp,
@@ -80,10 +57,8 @@ k_nfn(int n, int npad, int nparts, const double* __restrict__ X, const double* _
   }
   if (stop) return;
   int* tie = flags;
-  __shared__ float sx[kBT], sy[kBT], sz[kBT], se[kBT];
-  __shared__ int sc[kBT];
-  __shared__ int slist[kNfnList][kBT];
-  __shared__ int any;
+  __shared__ float4 sq[kBT];  // x, y, z and the component's bits
+  __shared__ int any, s_emax;
   const int i = blockIdx.x * kBT + threadIdx.x;
   const int part = blockIdx.y;
   bool need = false;
@@ -93,70 +68,87 @@ k_nfn(int n, int npad, int nparts, const double* __restrict__ X, const double* _
     const int b = nbr[i];
     need = (b < 0) || (comp[b] == ci);
   }
-  if (threadIdx.x == 0) any = 0;
+  if (threadIdx.x == 0) {
+    any = 0;
+    s_emax = 0;
+  }
   __syncthreads();
   if (need) any = 1;
   __syncthreads();
   if (!any) return;
-  const float xi = i < n ? f4[4 * i] : 0.0f, yi = i < n ? f4[4 * i + 1] : 0.0f, zi = i < n ? f4[4 * i + 2] : 0.0f;
-  const float ei = i < n ? f4[4 * i + 3] : 0.0f;
+  const float4* f = reinterpret_cast<const float4*>(f4);
+  const float4 fi = i < n ? f[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   const int per = (n + nparts - 1) / nparts;
   const int j_lo = part * per, j_hi = min(n, j_lo + per);
-  float bhi = __int_as_float(0x7f800000);
-  int listed = 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int t0 = j_lo; t0 < j_hi; t0 += kBT) {
-      __syncthreads();
-      const int j = t0 + threadIdx.x;
-      if (j < j_hi) {
-        sx[threadIdx.x] = f4[4 * j];
-        sy[threadIdx.x] = f4[4 * j + 1];
-        sz[threadIdx.x] = f4[4 * j + 2];
-        se[threadIdx.x] = f4[4 * j + 3];
-        sc[threadIdx.x] = comp[j];
-      }
-      __syncthreads();
-      if (!need) continue;
-      const int cnt = min(kBT, j_hi - t0);
-      if (pass == 0) {
-        for (int q = 0; q < cnt; ++q) {
-          const float h = d2_upper(fabsf(xi - sx[q]), fabsf(yi - sy[q]), fabsf(zi - sz[q]), ei + se[q]);
-          if (sc[q] != ci) bhi = fminf(bhi, h);
-        }
-      } else {
-        for (int q = 0; q < cnt; ++q) {
-          const float lo = d2_lower(fabsf(xi - sx[q]), fabsf(yi - sy[q]), fabsf(zi - sz[q]), ei + se[q]);
-          if (lo <= bhi && sc[q] != ci) {
-            if (listed < kNfnList) slist[listed][threadIdx.x] = t0 + q;
-            ++listed;
-          }
-        }
-      }
+  NearestScan ns;
+  ns.clear();
+  for (int t0 = j_lo; t0 < j_hi; t0 += kBT) {
+    __syncthreads();
+    const int j = t0 + threadIdx.x;
+    float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (j < j_hi) {
+      q = f[j];
+      sq[threadIdx.x] = make_float4(q.x, q.y, q.z, __int_as_float(comp[j]));
+    }
+    const int e = __reduce_max_sync(0xffffffffu, __float_as_int(q.w));  // non-negative floats
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_emax, e);
+    __syncthreads();
+    if (!need) continue;
+    const int cnt = min(kBT, j_hi - t0);
+#pragma unroll 4
+    for (int k = 0; k < cnt; ++k) {
+      const float4 c = sq[k];
+      ns.add(fi.x - c.x, fi.y - c.y, fi.z - c.z, __float_as_int(c.w) != ci, t0 + k);
     }
   }
-  if (!need) return;
+  __syncthreads();
+  const float emax = fi.w + __int_as_float(s_emax);
   unsigned long long bD = ~0ull;
   int bj = -1;
   int mytie = 0;
-  auto consider = [&](int jj) {
-    const unsigned long long db = key_bits(d2_exact(X, Y, Z, i, jj));
-    if (db < bD) {
-      bD = db;
-      bj = jj;
-    } else if (db == bD && jj != bj) {
-      mytie = 1;
+  const bool found = need && !ns.none();  // (a slice may hold no vertex of another component)
+  const bool sure = !found || ns.certain(emax);
+  if (found && sure) {
+    bj = ns.j1;
+    bD = key_bits(d2_exact(X, Y, Z, i, bj));
+  }
+  // the undecided vertices of the warp, one at a time over its 32 lanes
+  const int lane = threadIdx.x & 31;
+  for (unsigned todo = __ballot_sync(0xffffffffu, !sure); todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const int vi = __shfl_sync(0xffffffffu, i, l), vc = __shfl_sync(0xffffffffu, ci, l);
+    const float lim = __shfl_sync(0xffffffffu, ns.limit(emax), l);
+    const float vx = __shfl_sync(0xffffffffu, fi.x, l), vy = __shfl_sync(0xffffffffu, fi.y, l),
+                vz = __shfl_sync(0xffffffffu, fi.z, l);
+    unsigned long long d = ~0ull;
+    int dj = -1, tied = 0;
+    for (int jj = j_lo + lane; jj < j_hi; jj += 32) {
+      if (comp[jj] == vc) continue;
+      const float4 c = f[jj];
+      const float dx = vx - c.x, dy = vy - c.y, dz = vz - c.z;
+      if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) > lim) continue;
+      const unsigned long long db = key_bits(d2_exact(X, Y, Z, vi, jj));
+      if (db < d) {
+        d = db;
+        dj = jj;
+        tied = 0;
+      } else if (db == d) {
+        tied = 1;
+      }
     }
-  };
-  if (listed <= kNfnList) {
-    for (int k = 0; k < listed; ++k) consider(slist[k][threadIdx.x]);
-  } else {
-    for (int jj = j_lo; jj < j_hi; ++jj) {
-      if (comp[jj] == ci) continue;
-      const float lo = d2_lower(fabsf(xi - f4[4 * jj]), fabsf(yi - f4[4 * jj + 1]), fabsf(zi - f4[4 * jj + 2]),
-                                ei + f4[4 * jj + 3]);
-      if (lo <= bhi) consider(jj);
+    const unsigned mh = __reduce_min_sync(0xffffffffu, (unsigned)(d >> 32));
+    const unsigned ml = __reduce_min_sync(0xffffffffu, (unsigned)(d >> 32) == mh ? (unsigned)d : ~0u);
+    const unsigned long long dm = ((unsigned long long)mh << 32) | ml;
+    const unsigned at = __ballot_sync(0xffffffffu, d == dm && dj >= 0);
+    const unsigned tb = __ballot_sync(0xffffffffu, d == dm && tied != 0);
+    const int j0 = __shfl_sync(0xffffffffu, dj, at ? __ffs(at) - 1 : 0);
+    if (lane == l && at) {
+      bD = dm;
+      bj = j0;
+      mytie = tb != 0 || (at & (at - 1)) != 0;
     }
   }
+  if (!need) return;
   partD[(size_t)part * npad + i] = bD;
   partJ[(size_t)part * npad + i] = bj;
   if (mytie) atomicOr(tie, 1);
