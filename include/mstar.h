@@ -306,7 +306,7 @@ MSTAR_API long long mstar_batch_launch_count(const mstar_batch* b);
 MSTAR_API void mstar_batch_free(mstar_batch* b);
 
 /* Largest n that mstar_accelerations_noalloc accepts. Its scratch is a fixed static device
-   array of about 1.1 MB (positions, masses and the per-tile partial sums for 2048 bodies). */
+   array of about 0.8 MB (the per-tile partial sums for 2048 bodies). */
 #define MSTAR_NOALLOC_MAX_N 2048
 
 /* No counterpart in the paper: an allocation-free form of the pair loop, for callers that
@@ -316,8 +316,8 @@ MSTAR_API void mstar_batch_free(mstar_batch* b);
    routine (no cudaMalloc/cudaFree, no allocating library call).
    Computes, with every pair taken as far (Cartesian separations, as n_d = 0), the
    accelerations a_i = G sum_j m_j (r_j - r_i)/|r_j - r_i|^3 and the force function
-   U = G sum_{i<j} m_i m_j / |r_j - r_i|. Its own kernel (128-body tiles, an FP64 reciprocal
-   square root, a plain FP64 sum of U) is not the context's pair kernel: the results agree
+   U = G sum_{i<j} m_i m_j / |r_j - r_i|. Its own kernel (tiles of 32, 64 or 128 bodies by n;
+   masses of any sign) is not the context's pair kernel: the results agree
    with mstar_accelerations on a context created with n_d = 0 to rounding (1e-13 relative),
    not bit for bit, since the reduction order and the scalar arithmetic differ.
    Arguments: n in [2, MSTAR_NOALLOC_MAX_N] (larger n: MSTAR_ERR_UNSUPPORTED); m[n] and

@@ -52,7 +52,7 @@
 // which reads their partials from L2 right after, so that no reduction trails the launch.
 #include "device.cuh"
 #include "internal.h"
-#include "pairint.cuh"
+#include "pairtile.cuh"
 
 namespace mstar {
 namespace {
@@ -131,52 +131,6 @@ __device__ __forceinline__ void near_block(int n, int npad, int slot, int n_d, c
   o[3 * (size_t)npad] = acc.u;
 }
 
-// The near and invalid pairs of a sub-tile pair as one bit per step: bit k of lane l's word is
-// set when body i must not meet j-slot (l + k) mod 32 of the sub-tile. near_row: the tree's near
-// partners of body i among those 32 (k_near_words; null: none are masked); cnt: bodies of the
-// sub-tile below n; self: the sub-tile is the warp's own (each pair once: step 16 for half the
-// lanes).
-__device__ __forceinline__ unsigned mask_word(const unsigned* near_row, bool i_pad, int cnt, bool self, int lane) {
-  unsigned w = near_row ? *near_row : 0u;
-  if (cnt < 32) w |= cnt > 0 ? ~0u << cnt : ~0u;
-  w = __funnelshift_r(w, w, lane);
-  if (self && lane >= 16) w |= 1u << 16;
-  return i_pad ? ~0u : w;
-}
-
-// Floats ordered as signed integers, for the warp-wide minima and maxima.
-__device__ __forceinline__ int float_key(float f) {
-  const int b = __float_as_int(f);
-  return b ^ ((b >> 31) & 0x7fffffff);
-}
-__device__ __forceinline__ float key_float(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
-
-// Common scale of a tile pair for the integer pair arithmetic (pairint.cuh).
-struct FixWindow {
-  bool ok;        // the tile pair can be taken in integers
-  int u;          // unit 2^u of the positions
-  int em;         // every mass < 2^em
-  float inv_max;  // 1 / r^2 limit: pairs closer than 2^-10 of the extent are not taken
-};
-
-// From the extents lo[3], hi[3] of the two tiles' bodies and their largest mass exponent. The
-// float copies of the positions err by 2^-24 of the largest coordinate, which must not exceed
-// 2^8 extents, so a float r^2 of a pair at the limit is within 12 % (the limit allows for 30 %).
-__device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi, int em, bool ok) {
-  FixWindow w;
-  const float ext = fmaxf(hi[0] - lo[0], fmaxf(hi[1] - lo[1], hi[2] - lo[2])) * (1.0f + 0x1p-18f);
-  float big = 0.0f;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) big = fmaxf(big, fmaxf(fabsf(lo[c]), fabsf(hi[c])));
-  w.ok = ok && ext >= 0x1p-30f && big <= 256.0f * ext;
-  const int E = (int)((__float_as_uint(ext) >> 23) & 255u) - 126;  // ext < 2^E
-  w.u = E - 62;
-  w.em = em;
-  const float r = ext * 0x1p-10f;
-  w.inv_max = 1.0f / (1.3f * r * r);
-  return w;
-}
-
 // 24 warps per SM (80 registers, 100 bytes spilt outside the pair loops): attempts at N = 10002
 // took 31.5, 31.3, 30.5 and 30.4 ms with 16, 20, 24 and 28.
 template <int W>
@@ -210,17 +164,22 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int j0 = J * T;
   const int i = I * T + tid;
-  const double xi = rx[i], yi = ry[i], zi = rz[i];
-  const double xj0 = rx[j0 + tid], yj0 = ry[j0 + tid], zj0 = rz[j0 + tid];
-  sx[tid] = xj0;
-  sy[tid] = yj0;
-  sz[tid] = zj0;
-  // masses as m 2^e with m in [2^62, 2^63)
-  MassSplit msi = mass_split(m[i]), msj = mass_split(m[j0 + tid]);
-  msi.m >>= 1;
-  msi.e += 1;
-  msj.m >>= 1;
-  msj.e += 1;
+  const double pi3[3] = {rx[i], ry[i], rz[i]};
+  const double pj3[3] = {rx[j0 + tid], ry[j0 + tid], rz[j0 + tid]};
+  const double mi = m[i], mj = m[j0 + tid], m0 = m[I * T];
+  const bool i_pad = i >= n;
+  const bool diag = (I == J);
+  bool eq;  // all masses of the tile pair are equal
+  const FixWindow fw = tile_window<W>(pi3, pj3, mi, mj, i_pad, j0 + tid >= n, m0, sbox, &eq);
+  sx[tid] = pj3[0];
+  sy[tid] = pj3[1];
+  sz[tid] = pj3[2];
+  sfx[tid] = fix_of(pj3[0], fw.u);
+  sfy[tid] = fix_of(pj3[1], fw.u);
+  sfz[tid] = fix_of(pj3[2], fw.u);
+  sf[tid] = make_float4(__double2float_rn(pj3[0]), __double2float_rn(pj3[1]), __double2float_rn(pj3[2]),
+                        __double2float_rn(mj));
+  const MassSplit msj = fix_mass(mj);
   smm[tid] = msj.m;
   sme[tid] = msj.e;
 #pragma unroll
@@ -229,207 +188,21 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
     say[w][tid] = 0.0;
     saz[w][tid] = 0.0;
   }
-  const bool i_pad = i >= n;
-  const float fx = __double2float_rn(xi), fy = __double2float_rn(yi), fz = __double2float_rn(zi);
-  const float fm = __double2float_rn(m[i]);
-  sf[tid] = make_float4(__double2float_rn(xj0), __double2float_rn(yj0), __double2float_rn(zj0),
-                        __double2float_rn(m[j0 + tid]));
-  double axi = 0.0, ayi = 0.0, azi = 0.0, uii = 0.0;
-  UAcc uacc;          // sum over j of m_j / r_ij of the pairs taken in the mixed arithmetic
-  bool ubad = false;  // a coincident pair: the force is undefined
-  const bool diag = (I == J);
-
-  // the tile pair's extent and mass range over its bodies below n (the window of fix_pair)
-  FixWindow fw;
-  bool eq;  // all its masses are equal
-  const double m0 = m[I * T];
-  {
-    const bool j_pad = j0 + tid >= n;
-    const float kInf = __int_as_float(0x7f800000);
-    float lo[3], hi[3];
-    const double pi3[3] = {xi, yi, zi}, pj3[3] = {xj0, yj0, zj0};
-    bool ok = true;
-    int em = -4096;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      lo[c] = fminf(i_pad ? kInf : __double2float_rd(pi3[c]), j_pad ? kInf : __double2float_rd(pj3[c]));
-      hi[c] = fmaxf(i_pad ? -kInf : __double2float_ru(pi3[c]), j_pad ? -kInf : __double2float_ru(pj3[c]));
-      ok &= (i_pad || fabs(pi3[c]) < 0x1p50) && (j_pad || fabs(pj3[c]) < 0x1p50);  // false for NaN
-    }
-    // masses within 2^-40 ... 2^40, so that the float bounds of m / r^2 neither overflow nor vanish
-    if (!i_pad) em = msi.e + 63;
-    if (!j_pad) em = max(em, msj.e + 63);
-    ok &= (i_pad || (msi.e + 63 > -40 && msi.e + 63 < 40)) && (j_pad || (msj.e + 63 > -40 && msj.e + 63 < 40));
-    eq = __all_sync(0xffffffffu, (i_pad || m[i] == m0) && (j_pad || m[j0 + tid] == m0));
-    ok = __all_sync(0xffffffffu, ok);
-    int key[7];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      key[c] = __reduce_min_sync(0xffffffffu, float_key(lo[c]));
-      key[3 + c] = __reduce_max_sync(0xffffffffu, float_key(hi[c]));
-    }
-    key[6] = __reduce_max_sync(0xffffffffu, em);
-    if constexpr (W > 1) {
-      if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) sbox[warp][c] = key[c];
-        sbox[warp][7] = (ok ? 1 : 0) | (eq ? 2 : 0);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          key[c] = min(key[c], sbox[w][c]);
-          key[3 + c] = max(key[3 + c], sbox[w][3 + c]);
-        }
-        key[6] = max(key[6], sbox[w][6]);
-        ok &= (sbox[w][7] & 1) != 0;
-        eq &= (sbox[w][7] & 2) != 0;
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      lo[c] = key_float(key[c]);
-      hi[c] = key_float(key[3 + c]);
-    }
-    fw = fix_window(lo, hi, key[6], ok);
-    // The three components of a force share one unit. Where this warp's bodies lie flat (the mean
-    // distance from the middle of the extent along one axis below an eighth of that along
-    // another), the small component would keep fewer bits than binary64 sums do: not taken.
-    const float sc = exp2f((float)(-(fw.u + 62))) * 0x1p16f;  // extent -> at most 2^16
-    unsigned dev[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float mid = 0.5f * (lo[c] + hi[c]);
-      const float di = i_pad ? 0.0f : fabsf(__double2float_rn(pi3[c]) - mid) * sc;
-      const float dj = j_pad ? 0.0f : fabsf(__double2float_rn(pj3[c]) - mid) * sc;
-      dev[c] = __reduce_add_sync(0xffffffffu, (unsigned)fminf(di + dj, 0x1p20f));
-    }
-    fw.ok &= 8u * min(dev[0], min(dev[1], dev[2])) >= max(dev[0], max(dev[1], dev[2]));
-  }
-  const long long fxi = fix_of(xi, fw.u), fyi = fix_of(yi, fw.u), fzi = fix_of(zi, fw.u);
-  sfx[tid] = fix_of(xj0, fw.u);
-  sfy[tid] = fix_of(yj0, fw.u);
-  sfz[tid] = fix_of(zj0, fw.u);
+  TileBody body;
+  body.set(pi3[0], pi3[1], pi3[2], mi, fw);
   __syncthreads();
 
 #pragma unroll 1
   for (int s = 0; s < W; ++s) {
     const int sub = (warp + s) & (W - 1);
     const bool self = diag && sub == warp;
-    if (!(diag && sub < warp)) {
-      const int kbeg = self ? 1 : 0;
-      const int kend = self ? 17 : 32;
-      const int js = sub * 32;
-      const unsigned mw = mask_word(near_words ? near_words + (size_t)(J * W + sub) * npad + i : nullptr, i_pad,
-                                    n - j0 - js, self, lane);
-      // Float bounds of the largest force on body i (fi) and, handed from lane to lane with the
-      // partners, on each j (fj), without the masses where they are equal; the closest pair decides
-      // whether integers serve.
-      float fi = 0.0f, fj = 0.0f, inv_hi = 0.0f;
-      if (fw.ok) {
-#pragma unroll 4
-        for (int k = kbeg; k < kend; ++k) {
-          const float4 q = sf[js + ((lane + k) & 31)];
-          const float dx = q.x - fx, dy = q.y - fy, dz = q.z - fz;
-          float inv = rcp_approx(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-          inv = (mw >> k) & 1u ? 0.0f : inv;
-          inv_hi = fmaxf(inv_hi, inv);
-          fi = fmaxf(fi, q.w * inv);
-          fj = fmaxf(fj, fm * inv);
-          fj = __shfl_sync(0xffffffffu, fj, (lane + 1) & 31);  // now of partner (lane + k + 1) mod 32
-        }
-        if (self) fj = __shfl_sync(0xffffffffu, fj, (lane + 15) & 31);  // steps 1 ... 16: partner lane + 17
-      }
-      if (__all_sync(0xffffffffu, fw.ok && inv_hi <= fw.inv_max)) {
-        if (eq) {
-          const float rm = rcp_approx(__double2float_rn(m0));
-          fi *= rm;
-          fj *= rm;
-        }
-        // accumulator units 2^L: forces below 2^58 units (the bounds hold within 1.5)
-        const int ei = (int)(__float_as_uint(1.5f * fi) >> 23) - 126, ej = (int)(__float_as_uint(1.5f * fj) >> 23) - 126;
-        const int Li = ei - 58, Lj = ej - 58, LU = (((eq ? 0 : fw.em) + ei + 1) >> 1) - 58;
-        const int jo = js + lane, wo = warp * 32 + lane;
-        const int cx = 116 + 2 * fw.u + (eq ? 64 : 0), ci = Li + cx, cu = LU + 60 + fw.u + (eq ? 64 : 0);
-        scj[wo] = Lj + cx;
-        sbx[wo] = 0;
-        sby[wo] = 0;
-        sbz[wo] = 0;
-        __syncwarp();
-        FixAcc ai{0, 0, 0};
-        unsigned long long ui = 16;  // the sum's shifts truncate: half a unit per term back
-        double si = exp2_int(Li), sj = exp2_int(Lj), su = exp2_int(LU);
-        if (eq) {
-#pragma unroll 2
-          for (int k = kbeg; k < kend; ++k) {
-            const int r = (lane + k) & 31, jl = js + r, wl = warp * 32 + r;
-            FixAcc aj{sbx[wl], sby[wl], sbz[wl]};
-            fix_pair_eq(fxi, fyi, fzi, sfx[jl], sfy[jl], sfz[jl], ci, scj[wl], cu, (mw >> k) & 1u, ai, aj, ui);
-            sbx[wl] = aj.x;
-            sby[wl] = aj.y;
-            sbz[wl] = aj.z;
-            __syncwarp();
-          }
-          si *= m0;
-          sj *= m0;
-          su *= m0;
-        } else {
-#pragma unroll 2
-          for (int k = kbeg; k < kend; ++k) {
-            const int r = (lane + k) & 31, jl = js + r, wl = warp * 32 + r;
-            FixAcc aj{sbx[wl], sby[wl], sbz[wl]};
-            fix_pair(fxi, fyi, fzi, sfx[jl], sfy[jl], sfz[jl], msi.m, msi.e, smm[jl], sme[jl], ci, scj[wl], cu,
-                     (mw >> k) & 1u, ai, aj, ui);
-            sbx[wl] = aj.x;
-            sby[wl] = aj.y;
-            sbz[wl] = aj.z;
-            __syncwarp();
-          }
-        }
-        const long long bias = eq ? 0 : (kend - kbeg) * kFixBias;
-        axi = fma((double)(ai.x - bias), si, axi);
-        ayi = fma((double)(ai.y - bias), si, ayi);
-        azi = fma((double)(ai.z - bias), si, azi);
-        uii = fma((double)ui, su, uii);
-        sax[warp][jo] = fma((double)(sbx[wo] - bias), sj, sax[warp][jo]);
-        say[warp][jo] = fma((double)(sby[wo] - bias), sj, say[warp][jo]);
-        saz[warp][jo] = fma((double)(sbz[wo] - bias), sj, saz[warp][jo]);
-        __syncwarp();
-      } else {
-#pragma unroll 2
-        for (int k = kbeg; k < kend; ++k) {
-          const int jl = js + ((lane + k) & 31);
-          const double xj = sx[jl], yj = sy[jl], zj = sz[jl];
-          const bool masked = (mw >> k) & 1u;
-          double dx = xj - xi, dy = yj - yi, dz = zj - zi;
-          // keep the separations in registers: recomputing them for the accumulations would
-          // cost three more FP64 instructions per pair
-          asm volatile("" : "+d"(dx), "+d"(dy), "+d"(dz));
-          unsigned long long Rn;
-          int eR;
-          double sj, si;
-          const unsigned long long mjm = smm[jl] << 1;
-          const int mje = sme[jl] - 1;
-          pair_scalars_core(dx, dy, dz, MassSplit{mjm, mje}, MassSplit{msi.m << 1, msi.e - 1}, Rn, eR, sj, si);
-          // masked pairs contribute nothing (integer selects on the bit patterns)
-          sj = __longlong_as_double(masked ? 0ll : __double_as_longlong(sj));
-          si = __longlong_as_double(masked ? 0ll : __double_as_longlong(si));
-          ubad |= !masked && Rn == 0ull;
-          // m_j / r = mjm Rn 2^(mje + eR) ~ hi64(mjm Rn) 2^(mje + eR + 64)
-          uacc.add(masked ? 0ull : __umul64hi(mjm, Rn), masked ? uacc.L : mje + eR + 64);
-          axi = fma(sj, dx, axi);
-          ayi = fma(sj, dy, ayi);
-          azi = fma(sj, dz, azi);
-          // j-side sums are kept with the opposite sign and negated once when written
-          sax[warp][jl] = fma(si, dx, sax[warp][jl]);
-          say[warp][jl] = fma(si, dy, say[warp][jl]);
-          saz[warp][jl] = fma(si, dz, saz[warp][jl]);
-          __syncwarp();
-        }
-      }
-    }
+    if (diag && sub < warp) continue;
+    const int js = sub * 32, wo = warp * 32;
+    const unsigned mw = mask_word(near_words ? near_words + (size_t)(J * W + sub) * npad + i : nullptr, i_pad,
+                                  n - j0 - js, self, lane);
+    const SubTile t{sx + js,  sy + js,  sz + js,       sfx + js,      sfy + js,      sfz + js, smm + js, sme + js,
+                    sf + js,  nullptr, &sax[warp][js], &say[warp][js], &saz[warp][js], sbx + wo,      sby + wo, sbz + wo, scj + wo};
+    subtile_pairs<false>(body, t, fw, eq, m0, mw, self ? 1 : 0, self ? 17 : 32, lane);
   }
   __syncthreads();
   // the warps' partner sums, in warp order
@@ -441,7 +214,7 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
     jz += saz[w][tid];
   }
 
-  const double ui = ubad ? __longlong_as_double(0x7ff8000000000000LL) : uii + uacc.value();
+  const double axi = body.ax, ayi = body.ay, azi = body.az, ui = body.u_sum();
   double* Ps = P + (size_t)slot * NT * 4 * npad;
   if (diag) {
     double* q = Ps + (size_t)I * 4 * npad + i;
