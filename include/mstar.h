@@ -79,10 +79,10 @@ typedef struct {
   int mst_nsub;      /* subgraphs of the divide-and-conquer octree, 0 = ceil(sqrt(n)), at most
                         1024. 0 */
   int pair_tile;     /* bodies per tile of the pair loop: 32, 64 or 128, or 0 for the size rule
-                        (32 up to 4096 bodies, 64 up to 8192, 128 above); mstar_tune_pair_tile
+                        (32 up to 8192 bodies, 128 above); mstar_tune_pair_tile
                         times the choices on a given system. 0 */
   int pair_split;    /* warps that share the 32 partner steps of a tile pair, with 32-body tiles:
-                        1, 2, 4 or 8, or 0 for the size rule (4 up to 512 bodies, else 1); the
+                        1, 2, 4 or 8, or 0 for the size rule (4 up to 768 bodies, else 1); the
                         other tiles take 1. Partial sums are added in warp order, so results
                         differ from the unsplit loop by rounding only. 0 */
   int division_schedule; /* how an attempt's k_fix divisions are issued: 1 level by level (the

@@ -56,7 +56,7 @@ Shape shape_of(int n, const mstar_params& p) {
   s.K = p.k_fix;
   s.S = p.k_fix + 1;
   s.NT = s.npad / s.T;
-  s.split = s.W != 1 ? 1 : (p.pair_split ? p.pair_split : (n <= 512 ? 4 : 1));
+  s.split = s.W != 1 ? 1 : (p.pair_split ? p.pair_split : (n <= 768 ? 4 : 1));
   s.nblk = (s.npad + kBlock - 1) / kBlock;
   s.dcb = p.mst_method == 1 ? dc_scratch_bytes(n, p.mst_nsub) : 0;
   return s;
@@ -545,12 +545,13 @@ int vectors_out(mstar_ctx* c, const double* planes, double* dst) {
   return MSTAR_OK;
 }
 
-// Pair tile of 32 W bodies by system size, from a sweep of full GBS steps on Plummer spheres
-// (pair-forces/s): below ~4000 bodies the 32-body tiles give the most CTAs per slot (+18 %
-// at N = 2050 over 128-body tiles); up to ~8000 the 64-body tiles; above, the 128-body
-// tiles keep the partial sums (slots x tiles x 4 x npad doubles) a quarter as large at the
-// same speed.
-int choose_tile_warps(int n) { return n <= 4096 ? 1 : (n <= 8192 ? 2 : 4); }
+// Pair tile of 32 W bodies by system size, from a sweep of full GBS steps on Plummer spheres. One
+// warp per CTA waits for no other: W = 1, 2, 4 take 5.26, 5.43, 5.43 ms at N = 4096, 7.75, 8.23, 8.47
+// at 5003, 18.8, 19.6, 19.3 at 8000 and 29.5, 30.8, 30.0 at 10002. Above 8192 the 128-body tiles
+// keep the partial sums (slots x tiles x 4 x npad doubles, 604 MB at N = 8192 with 32-body tiles) a
+// quarter as large for 2 % of the speed. Up to 768 bodies a tile pair's steps are split over four
+// warps (pair_split 4; 0.91 against 0.93 ms at N = 601, equal at 800, 3 % slower at 900).
+int choose_tile_warps(int n) { return n <= 8192 ? 1 : 4; }
 
 size_t workspace_bytes(int n, const mstar_params& p, int* npad_out, int* W_out) {
   Shape s = shape_of(n, p);

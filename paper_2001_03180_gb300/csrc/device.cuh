@@ -201,44 +201,6 @@ struct NearAcc {
   }
 };
 
-// The near pairs of body p (Sec. 3.4, N_d <= 2: parent, children, grandparent, grandchildren,
-// siblings), each from the edge vectors X (3 planes) summed along the tree path between the
-// two bodies, added to acc.
-__device__ __forceinline__ void near_terms(int p, int npad, int n_d, const double* __restrict__ X,
-                                           const double* __restrict__ m, const int* __restrict__ parent,
-                                           const int* __restrict__ gp, const int* __restrict__ child_off,
-                                           const int* __restrict__ child_idx, NearAcc& acc) {
-  if (n_d < 1) return;
-  const double* Xx = X;
-  const double* Xy = Xx + npad;
-  const double* Xz = Xy + npad;
-  const int pp = parent[p];
-  const double xp = Xx[p], yp = Xy[p], zp = Xz[p];
-  if (pp >= 0) acc.add(p, pp, -xp, -yp, -zp, m[pp]);
-  const int c0 = child_off[p], c1 = child_off[p + 1];
-  for (int a = c0; a < c1; ++a) {
-    const int c = child_idx[a];
-    acc.add(p, c, Xx[c], Xy[c], Xz[c], m[c]);
-  }
-  if (n_d < 2) return;
-  const int g = gp[p];
-  if (g >= 0) acc.add(p, g, -(xp + Xx[pp]), -(yp + Xy[pp]), -(zp + Xz[pp]), m[g]);
-  for (int a = c0; a < c1; ++a) {
-    const int c = child_idx[a];
-    const double xc = Xx[c], yc = Xy[c], zc = Xz[c];
-    for (int b = child_off[c]; b < child_off[c + 1]; ++b) {
-      const int gc = child_idx[b];
-      acc.add(p, gc, Xx[gc] + xc, Xy[gc] + yc, Xz[gc] + zc, m[gc]);
-    }
-  }
-  if (pp >= 0) {
-    for (int b = child_off[pp]; b < child_off[pp + 1]; ++b) {
-      const int sib = child_idx[b];
-      if (sib != p) acc.add(p, sib, Xx[sib] - xp, Xy[sib] - yp, Xz[sib] - zp, m[sib]);
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------------------
 // Exact sums of positive terms on the integer pipe.
 //

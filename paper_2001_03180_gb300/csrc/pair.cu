@@ -112,23 +112,101 @@ __device__ __forceinline__ void finish_tile(int t, int npad, int NT, const doubl
   if (tid == 0) cnt[t] = 0;
 }
 
-// The near pairs of Sec. 3.4 (N_d <= 2) of the CTA's bodies, one per thread, into Nb (4 planes:
-// ax, ay, az and the sum of m/r over partners of higher index). They depend on the slot's edge
-// vectors alone, so the pair launches take them in CTAs of their own ahead of the tile pairs,
-// and the finishing pass adds them to the tile sums instead of walking the near partners itself.
+// The near pairs of Sec. 3.4 (N_d <= 2) of the CTA's bodies, into Nb (4 planes: ax, ay, az and the
+// sum of m/r over partners of higher index). They depend on the slot's edge vectors alone, so the
+// pair launches take them in CTAs of their own ahead of the tile pairs, and the finishing pass adds
+// them to the tile sums instead of walking the near partners itself.
+//
+// L lanes share a body's partners: a walk by one lane is a chain of up to some 25 partners (the
+// largest counts in its warp), each an L2 access and a dependent 1/r^3, and bound the launches of
+// small systems (N = 256: 14.8 us a launch, 8.2 with eight lanes and k_pair_tiles_ks' integers). Where
+// the tile pairs fill the GPU the idle lanes' FP64 slots count instead: eight lanes cost 1 % of an
+// attempt at N = 5003.
+template <int S>
+constexpr int kNearLanes = S > 1 ? 8 : 1;
+template <int L>
 __device__ __forceinline__ void near_block(int n, int npad, int slot, int n_d, const double* __restrict__ m,
                                            const int* __restrict__ parent, const int* __restrict__ gp,
                                            const int* __restrict__ child_off, const int* __restrict__ child_idx,
                                            const double* __restrict__ sX, double* __restrict__ Nb) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int l = threadIdx.x & (L - 1);
+  const unsigned group = ((1u << L) - 1) << (threadIdx.x & 31 & ~(L - 1));
+  const int p = idx / L;
+  if (p >= n) return;  // whole groups
+  const double *Xx = sX + (size_t)slot * 3 * npad, *Xy = Xx + npad, *Xz = Xy + npad;
+  const bool nd2 = n_d >= 2;
+  const int pp = parent[p], g = nd2 ? gp[p] : -1, c0 = child_off[p], c1 = child_off[p + 1];
+  const int b0 = nd2 && pp >= 0 ? child_off[pp] : 0, b1 = nd2 && pp >= 0 ? child_off[pp + 1] : 0;
+  const double xp = Xx[p], yp = Xy[p], zp = Xz[p];
   NearAcc acc;
-  near_terms(p, npad, n_d, sX + (size_t)slot * 3 * npad, m, parent, gp, child_off, child_idx, acc);
+  // +x, -x or 0 (sign and keep masks): off the FP64 pipe
+  auto pick = [](double x, unsigned long long sign, unsigned long long keep) {
+    return __longlong_as_double((long long)(((unsigned long long)__double_as_longlong(x) ^ sign) & keep));
+  };
+  // parent, grandparent, children, siblings: the separation is the picked X_k plus -X_p or 0
+  for (int t = l; t < 2 + (c1 - c0) + (b1 - b0); t += L) {
+    int q, k;
+    constexpr unsigned long long kSign = 1ull << 63;
+    unsigned long long sign = 0ull, keep = ~0ull, keep_p = ~0ull;
+    if (t < 2) {
+      q = t == 0 ? pp : g;
+      k = pp;
+      sign = kSign;
+      keep = t == 0 ? 0ull : ~0ull;
+    } else if (t < 2 + (c1 - c0)) {
+      q = k = child_idx[c0 + t - 2];
+      keep_p = 0ull;
+    } else {
+      q = k = child_idx[b0 + t - 2 - (c1 - c0)];
+      if (q == p) q = -1;
+    }
+    if (q >= 0)
+      acc.add(p, q, pick(Xx[k], sign, keep) + pick(xp, kSign, keep_p), pick(Xy[k], sign, keep) + pick(yp, kSign, keep_p),
+              pick(Xz[k], sign, keep) + pick(zp, kSign, keep_p), m[q]);
+  }
+  if (nd2) {
+    // grandchildren, in the children's order: L children at a time
+    for (int a = c0; a < c1; a += L) {
+      const int c = a + l < c1 ? child_idx[a + l] : -1;
+      const int o = c >= 0 ? child_off[c] : 0, cnt = c >= 0 ? child_off[c + 1] - o : 0;
+      int inc = cnt;
+#pragma unroll
+      for (int d = 1; d < L; d <<= 1) {
+        const int v = __shfl_up_sync(group, inc, d, L);
+        inc += l >= d ? v : 0;
+      }
+      const int tot = __shfl_sync(group, inc, L - 1, L);
+      for (int t0 = 0; t0 < tot; t0 += L) {
+        const int t = t0 + l;
+        int k = 0;  // the child holding grandchild t
+#pragma unroll
+        for (int d = 0; d < L - 1; ++d) k += __shfl_sync(group, inc, d, L) <= t;
+        const int ck = __shfl_sync(group, c, k, L);
+        const int at = __shfl_sync(group, o - (inc - cnt), k, L) + t;
+        if (t < tot) {
+          const int q = child_idx[at];
+          acc.add(p, q, Xx[q] + Xx[ck], Xy[q] + Xy[ck], Xz[q] + Xz[ck], m[q]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int d = L / 2; d > 0; d >>= 1) {
+    acc.ax += __shfl_xor_sync(group, acc.ax, d);
+    acc.ay += __shfl_xor_sync(group, acc.ay, d);
+    acc.az += __shfl_xor_sync(group, acc.az, d);
+    acc.u += __shfl_xor_sync(group, acc.u, d);
+  }
   double* o = Nb + (size_t)slot * 4 * npad + p;
-  o[0] = acc.ax;
-  o[(size_t)npad] = acc.ay;
-  o[2 * (size_t)npad] = acc.az;
-  o[3 * (size_t)npad] = acc.u;
+  if constexpr (L >= 4) {
+    if (l < 4) o[(size_t)l * npad] = l == 0 ? acc.ax : (l == 1 ? acc.ay : (l == 2 ? acc.az : acc.u));
+  } else if (l == 0) {
+    o[0] = acc.ax;
+    o[(size_t)npad] = acc.ay;
+    o[2 * (size_t)npad] = acc.az;
+    o[3 * (size_t)npad] = acc.u;
+  }
 }
 
 // 24 warps per SM (80 registers, 100 bytes spilt outside the pair loops): attempts at N = 10002
@@ -153,7 +231,7 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
 
   const int slot = slot_lo + blockIdx.y;
   if ((int)blockIdx.x < nnear) {
-    near_block(n, npad, slot, n_d, m, parent, gp, child_off, child_idx, sX, Nb);
+    near_block<kNearLanes<1>>(n, npad, slot, n_d, m, parent, gp, child_off, child_idx, sX, Nb);
     return;
   }
   int I, J;
@@ -259,14 +337,16 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
   }
 }
 
-// The pair loop of small systems: the tiling and per-pair arithmetic of k_pair_tiles<1>
-// (32-body tiles), with the 32 partner steps of a tile pair split over S warps (S divides
-// 16). Warp w takes steps [32 w / S, 32 (w + 1) / S) of an off-diagonal pair and
-// [1 + 16 w / S, 1 + 16 (w + 1) / S) of a diagonal one, keeping its own i-side sums and its
-// own copy of the partner sums; the S copies are added in warp order at the end. At N ~ 10^2
-// a tile pair's 32 dependent steps in one warp bind the launch; S warps shorten them S-fold.
+// The pair loop of small systems: the 32-body tiles and the arithmetic of k_pair_tiles<1>, with the
+// 32 partner steps of a tile pair split over S warps (S divides 16). Warp w takes steps
+// [32 w / S, 32 (w + 1) / S) of an off-diagonal pair and [1 + 16 w / S, 1 + 16 (w + 1) / S) of a
+// diagonal one, keeping its own i-side and partner sums; the S copies are added in warp order at the
+// end. At N ~ 10^2 to 10^3 a tile pair's 32 dependent steps in one warp bind the launch; S warps
+// shorten them S-fold. What does not shrink is done once, by warp 0 (conversions and window: some
+// 500 cycles of FP64 pipe), or binds larger S (a warp's flush to FP64: 14 FP64 instructions).
+// Attempts with S = 1, 2, 4, 8: 0.83, 0.77, 0.73, 0.73 ms at N = 256, 0.80, 0.76, 0.73, 0.80 at 512.
 template <int S>
-__global__ void __launch_bounds__(32 * S)
+__global__ void __launch_bounds__(32 * S, 24 / S)
 k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __restrict__ m,
                 const int* __restrict__ parent, const int* __restrict__ gp, const double* __restrict__ sr,
                 double* __restrict__ P, double* __restrict__ Pt, int* __restrict__ tcnt, int keep_from,
@@ -274,13 +354,18 @@ k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __r
                 const double* __restrict__ sX, double* __restrict__ Nb, int nnear) {
   constexpr int T = 32;
   __shared__ double sx[T], sy[T], sz[T];
-  __shared__ double sax[S][T], say[S][T], saz[S][T];     // partner sums, one copy per warp
-  __shared__ double rax[S][T], ray[S][T], raz[S][T], rau[S][T];  // i-side sums per warp
+  __shared__ long long sfx[T], sfy[T], sfz[T];
   __shared__ unsigned long long smm[T];
-  __shared__ int sp[T], sg[T], sme[T];
+  __shared__ int sme[T], scj[S][T], sp[T], sg[T];
+  __shared__ float4 sf[T];
+  __shared__ TilePos sbody[T];
+  __shared__ FixWindow sfw;
+  __shared__ bool seq;
+  __shared__ double sj3[S][3][T];  // partner sums per warp
+  __shared__ double si4[S][4][T];  // integer sums of the partners, then the i-side sums per warp
   const int slot = slot_lo + blockIdx.y;
   if ((int)blockIdx.x < nnear) {
-    near_block(n, npad, slot, n_d, m, parent, gp, child_off, child_idx, sX, Nb);
+    near_block<kNearLanes<S>>(n, npad, slot, n_d, m, parent, gp, child_off, child_idx, sX, Nb);
     return;
   }
   int I, J;
@@ -289,98 +374,81 @@ k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __r
   const double* ry = rx + npad;
   const double* rz = ry + npad;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int j0 = J * T;
-  if (warp == 0) {
-    sx[lane] = rx[j0 + lane];
-    sy[lane] = ry[j0 + lane];
-    sz[lane] = rz[j0 + lane];
-    const MassSplit ms = mass_split(m[j0 + lane]);
+  const int j0 = J * T, i = I * T + lane, j = j0 + lane;
+  const bool i_pad = i >= n, diag = I == J;
+  const int pi = parent[i], gpi = gp[i];
+  const double m0 = m[I * T];
+  if (warp == 0) {  // the conversions once: FP64 pipe
+    const double pi3[3] = {rx[i], ry[i], rz[i]};
+    const double pj3[3] = {rx[j], ry[j], rz[j]};
+    const double mi = m[i], mj = m[j];
+    bool eq;
+    const FixWindow fw = tile_window<1>(pi3, pj3, mi, mj, i_pad, j >= n, m0, nullptr, &eq);
+    sx[lane] = pj3[0];
+    sy[lane] = pj3[1];
+    sz[lane] = pj3[2];
+    sfx[lane] = fix_of(pj3[0], fw.u);
+    sfy[lane] = fix_of(pj3[1], fw.u);
+    sfz[lane] = fix_of(pj3[2], fw.u);
+    sf[lane] = make_float4(__double2float_rn(pj3[0]), __double2float_rn(pj3[1]), __double2float_rn(pj3[2]),
+                           __double2float_rn(mj));
+    const MassSplit ms = fix_mass(mj);
     smm[lane] = ms.m;
     sme[lane] = ms.e;
-    sp[lane] = parent[j0 + lane];
-    sg[lane] = gp[j0 + lane];
+    sp[lane] = parent[j];
+    sg[lane] = gp[j];
+    TilePos b;
+    b.set(pi3[0], pi3[1], pi3[2], mi, fw);
+    sbody[lane] = b;
+    if (lane == 0) {
+      sfw = fw;
+      seq = eq;
+    }
   }
-  sax[warp][lane] = 0.0;
-  say[warp][lane] = 0.0;
-  saz[warp][lane] = 0.0;
-  const int i = I * T + lane;
-  const double xi = rx[i], yi = ry[i], zi = rz[i];
-  const MassSplit msi = mass_split(m[i]);
-  const int pi = parent[i], gpi = gp[i];
-  const bool i_pad = i >= n;
-  const bool nd1 = n_d >= 1, nd2 = n_d >= 2;
-  double axi = 0.0, ayi = 0.0, azi = 0.0;
-  UAcc uacc;
-  bool ubad = false;
-  const bool diag = (I == J);
-  const int kbeg = diag ? 1 + 16 * warp / S : 32 * warp / S;
-  const int kend = diag ? 1 + 16 * (warp + 1) / S : 32 * (warp + 1) / S;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) sj3[warp][c][lane] = 0.0;
   __syncthreads();
-#pragma unroll 4
-  for (int k = kbeg; k < kend; ++k) {
-    const int jl = (lane + k) & 31;
-    const int j = j0 + jl;
-    const double xj = sx[jl], yj = sy[jl], zj = sz[jl];
-    const int pj = sp[jl], gj = sg[jl];
-    bool masked = i_pad | (j >= n) | (diag & (k == 16) & (lane >= 16));
-    masked |= nd1 & ((pi == j) | (pj == i));
-    masked |= nd2 & ((gpi == j) | (gj == i) | (pi == pj));
-    double dx = xj - xi, dy = yj - yi, dz = zj - zi;
-    asm volatile("" : "+d"(dx), "+d"(dy), "+d"(dz));
-    unsigned long long Rn;
-    int eR;
-    double sj, si;
-    const unsigned long long mjm = smm[jl];
-    const int mje = sme[jl];
-    pair_scalars_core(dx, dy, dz, MassSplit{mjm, mje}, msi, Rn, eR, sj, si);
-    sj = __longlong_as_double(masked ? 0ll : __double_as_longlong(sj));
-    si = __longlong_as_double(masked ? 0ll : __double_as_longlong(si));
-    ubad |= !masked && Rn == 0ull;
-    uacc.add(masked ? 0ull : __umul64hi(mjm, Rn), masked ? uacc.L : mje + eR + 64);
-    axi = fma(sj, dx, axi);
-    ayi = fma(sj, dy, ayi);
-    azi = fma(sj, dz, azi);
-    sax[warp][jl] = fma(si, dx, sax[warp][jl]);
-    say[warp][jl] = fma(si, dy, say[warp][jl]);
-    saz[warp][jl] = fma(si, dz, saz[warp][jl]);
-    __syncwarp();
+  TileBody body;
+  static_cast<TilePos&>(body) = sbody[lane];
+  const FixWindow fw = sfw;
+  const bool eq = seq;
+  {
+    long long* sb = reinterpret_cast<long long*>(&si4[warp][0][0]);
+    const SubTile t{sx,           sy,           sz,           sfx, sfy,    sfz,    smm,      sme, sf, nullptr,
+                    sj3[warp][0], sj3[warp][1], sj3[warp][2], sb,  sb + 32, sb + 64, scj[warp]};
+    const int k0 = diag ? 1 + 16 * warp / S : 32 * warp / S, k1 = k0 + (diag ? 16 : 32) / S;
+    // the near pairs of the warp's few steps, here (a pass of its own over the tree would cost
+    // small systems a launch)
+    unsigned mw = mask_word(nullptr, i_pad, n - j0, diag, lane);
+    if (n_d >= 1)
+      for (int k = k0; k < k1; ++k) {
+        const int q = (lane + k) & 31, jq = j0 + q, pj = sp[q];
+        bool near = (pi == jq) | (pj == i);
+        near |= (n_d >= 2) & ((gpi == jq) | (sg[q] == i) | (pi == pj));
+        mw |= near ? 1u << k : 0u;
+      }
+    subtile_pairs<false>(body, t, fw, eq, m0, mw, k0, k1, lane);
   }
-  rax[warp][lane] = axi;
-  ray[warp][lane] = ayi;
-  raz[warp][lane] = azi;
-  rau[warp][lane] = ubad ? __longlong_as_double(0x7ff8000000000000LL) : uacc.value();
+  __syncwarp();
+  si4[warp][0][lane] = body.ax;
+  si4[warp][1][lane] = body.ay;
+  si4[warp][2][lane] = body.az;
+  si4[warp][3][lane] = body.u_sum();
   __syncthreads();
+  // warp c (round robin) adds component c of the S copies
   double* Ps = P + (size_t)slot * NT * 4 * npad;
-  if (warp == 0) {
-    double ax = rax[0][lane], ay = ray[0][lane], az = raz[0][lane], u = rau[0][lane];
-    double jx = sax[0][lane], jy = say[0][lane], jz = saz[0][lane];
+  for (int c = warp; c < 4; c += S) {
+    double a = si4[0][c][lane], jv = c < 3 ? sj3[0][c][lane] : 0.0;
 #pragma unroll
     for (int w = 1; w < S; ++w) {
-      ax += rax[w][lane];
-      ay += ray[w][lane];
-      az += raz[w][lane];
-      u += rau[w][lane];
-      jx += sax[w][lane];
-      jy += say[w][lane];
-      jz += saz[w][lane];
+      a += si4[w][c][lane];
+      if (c < 3) jv += sj3[w][c][lane];
     }
     if (diag) {
-      double* q = Ps + (size_t)I * 4 * npad + i;
-      q[0] = ax - jx;
-      q[(size_t)npad] = ay - jy;
-      q[2 * (size_t)npad] = az - jz;
-      q[3 * (size_t)npad] = u;
+      Ps[(size_t)I * 4 * npad + (size_t)c * npad + i] = a - jv;
     } else {
-      double* q = Ps + (size_t)J * 4 * npad + i;
-      q[0] = ax;
-      q[(size_t)npad] = ay;
-      q[2 * (size_t)npad] = az;
-      q[3 * (size_t)npad] = u;
-      double* qj = Ps + (size_t)I * 4 * npad + j0 + lane;
-      qj[0] = -jx;
-      qj[(size_t)npad] = -jy;
-      qj[2 * (size_t)npad] = -jz;
-      qj[3 * (size_t)npad] = 0.0;
+      Ps[(size_t)J * 4 * npad + (size_t)c * npad + i] = a;
+      Ps[(size_t)I * 4 * npad + (size_t)c * npad + j] = -jv;
     }
   }
   // the on-chip reduction of k_pair_tiles (the first 32 threads sum a tile)
@@ -516,7 +584,7 @@ int defer_slots(const mstar_ctx* c, K kernel, int threads) {
 template <int W, int S>
 cudaError_t run_tiles(mstar_ctx* c, int slot_lo, int nsl, int n_d, int keep_from) {
   constexpr int threads = S == 1 ? 32 * W : 32 * S;
-  const int nnear = n_d >= 1 ? (c->n + threads - 1) / threads : 0;  // the near CTAs come first
+  const int nnear = n_d >= 1 ? (c->n * kNearLanes<S> + threads - 1) / threads : 0;  // the near CTAs come first
   dim3 grid(nnear + c->ntp, nsl);
   if (c->prof) prof_begin(c);
   if constexpr (S == 1)

@@ -135,15 +135,12 @@ __device__ __forceinline__ MassSplit fix_mass(double m) {
   return s;
 }
 
-// The lane's body of the i side, and its sums over the partners met so far.
-struct TileBody {
+// The lane's body of the i side.
+struct TilePos {
   double x, y, z, m;     // m: read by the plain fallback only
   long long fx, fy, fz;  // fixed point
   float gx, gy, gz, gm;  // float copies
   MassSplit ms;          // fix_mass
-  double ax = 0.0, ay = 0.0, az = 0.0, u = 0.0;
-  UAcc uacc;             // sum of m_j / r_ij of the pairs taken in the mixed arithmetic
-  bool bad = false;      // a coincident pair: the force is undefined
   __device__ __forceinline__ void set(double x_, double y_, double z_, double m, const FixWindow& w) {
     fx = fix_of(x_, w.u);
     fy = fix_of(y_, w.u);
@@ -158,6 +155,13 @@ struct TileBody {
     z = z_;
     this->m = m;
   }
+};
+
+// The same with its sums over the partners met so far.
+struct TileBody : TilePos {
+  double ax = 0.0, ay = 0.0, az = 0.0, u = 0.0;
+  UAcc uacc;             // sum of m_j / r_ij of the pairs taken in the mixed arithmetic
+  bool bad = false;      // a coincident pair: the force is undefined
   __device__ __forceinline__ double u_sum() const {
     return bad ? __longlong_as_double(0x7ff8000000000000LL) : u + uacc.value();
   }

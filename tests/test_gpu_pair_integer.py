@@ -66,6 +66,41 @@ def test_both_arithmetics_match_the_oracle(n, tile, kind, n_d):
     assert abs(U - Uo) <= tol * pot
 
 
+@pytest.mark.parametrize("n,split", [(45, 2), (200, 0), (513, 8), (900, 0)])
+@pytest.mark.parametrize("n_d", [1, 2])
+def test_near_pairs_of_a_node_of_high_degree(n, split, n_d):
+    """A body with 12 tree neighbours (the centre of an icosahedron, whose edges are 5 % longer than
+    its radius), some with children of their own: more partners than share lanes. Same tolerance."""
+    m, r, v = W.plummer(n, 17)
+    r = r + 20.0
+    g = (1.0 + 5.0 ** 0.5) / 2.0
+    ico = np.array([(0, a, b * g) for a in (-1, 1) for b in (-1, 1)], float)
+    ico = np.concatenate([ico, ico[:, [1, 2, 0]], ico[:, [2, 0, 1]]]) * (1.0 + 1e-3 * np.arange(12))[:, None]
+    r[0] = 0.0
+    r[1:13] = ico
+    r[13:25] = 1.4 * ico
+    r[25:34] = 1.5 * ico[:9] + 0.1
+    it = M.Integrator(m, r, v, n_d=n_d, pair_split=split)
+    a, U = it.accelerations()
+    rs = it.state()["r"]
+    it.close()
+    root, par, lev, order = O.prim(rs)
+    deg = np.bincount(par[par >= 0], minlength=n) + (par >= 0)
+    assert deg.max() >= 12
+    ao, Uo = O.forces(m, rs, par, lev, O.to_mst(par, rs), n_d=n_d)
+    d = rs[None, :, :] - rs[:, None, :]
+    dist = np.sqrt((d * d).sum(-1))
+    np.fill_diagonal(dist, np.inf)
+    terms = (m[None, :, None] * np.abs(d) / dist[..., None] ** 3).sum(1)
+    pot = 0.5 * (m[:, None] * m[None, :] / dist).sum()
+    tol = 2.0 * (n + 8) * 2.0 ** -53
+    # both sides take near separations from the same kind of path sums; their own rounding (3 sums of
+    # coordinates below 50 over distances above 0.1) is not the oracle's: 3 * 500 u on each term
+    tol += 2 * 3 * 500 * 2.0 ** -53
+    assert (np.abs(a - ao) <= tol * np.maximum(terms, 1e-300)).all(), (np.abs(a - ao) / terms).max() / tol
+    assert abs(U - Uo) <= tol * pot
+
+
 def test_a_coincident_far_pair_is_undefined():
     """Two coincident bodies that are not tree neighbours: U and both accelerations are NaN, the
     others finite, as in the mixed arithmetic alone."""
