@@ -252,17 +252,15 @@ k_prim(int n, int npad, const double* __restrict__ r, int* __restrict__ parent_o
     cw.l1 = __reduce_min_sync(0xffffffffu, c.l1);
     cw.l1idx = (int)__reduce_min_sync(0xffffffffu, c.l1 == cw.l1 ? (unsigned)c.l1idx : 0xffffffffu);
     cw.l2 = __reduce_min_sync(0xffffffffu, (c.l1 == cw.l1 && c.l1idx == cw.l1idx) ? c.l2 : c.l1);
-    if (nw > 1) {
-      if (lane == 0) rc[warp] = cw;
-      __syncthreads();
-      if (warp == 0) {
-        cw = lane < nw ? rc[lane] : cand_identity();
-        for (int o = 16; o > 0; o >>= 1) cand_combine(cw, cand_shfl_down(cw, o));
-        if (lane == 0) wc = cw;
-      }
-      __syncthreads();
-      cw = wc;
+    if (lane == 0) rc[warp] = cw;
+    __syncthreads();
+    if (warp == 0) {
+      cw = lane < nw ? rc[lane] : cand_identity();
+      for (int o = 16; o > 0; o >>= 1) cand_combine(cw, cand_shfl_down(cw, o));
+      if (lane == 0) wc = cw;
     }
+    __syncthreads();
+    cw = wc;
     int nxt;
     if (cw.l1idx == cw.hidx && cw.l2 > cw.hk) {
       nxt = cw.hidx;
@@ -302,6 +300,151 @@ k_prim(int n, int npad, const double* __restrict__ r, int* __restrict__ parent_o
   for (int w = tid; w < n; w += nt) {
     parent_out[w] = par[w];
     level_out[w] = lvl[w];
+  }
+}
+
+// The float interval of d(u,w)^2 that k_prim derives, for vertices (x, y, z).
+__device__ __forceinline__ void d2_interval(float4 u, float4 w, float& lo, float& hi) {
+  const float ax = fabsf(u.x - w.x), ay = fabsf(u.y - w.y), az = fabsf(u.z - w.z);
+  const float ex = (fabsf(u.x) + fabsf(w.x) + ax) * 0x1p-23f + 1e-37f;
+  const float ey = (fabsf(u.y) + fabsf(w.y) + ay) * 0x1p-23f + 1e-37f;
+  const float ez = (fabsf(u.z) + fabsf(w.z) + az) * 0x1p-23f + 1e-37f;
+  const float lx = fmaxf(ax - ex, 0.0f), ly = fmaxf(ay - ey, 0.0f), lz = fmaxf(az - ez, 0.0f);
+  const float hx = ax + ex, hy = ay + ey, hz = az + ez;
+  lo = fmaxf(((lx * lx + ly * ly) + lz * lz) * (1.0f - 0x1p-20f) - 0x1p-144f, 0.0f);
+  hi = ((hx * hx + hy * hy) + hz * hz) * (1.0f + 0x1p-20f);
+}
+
+// k_prim for at most kPrimSmallN bodies: the same keys and decisions, for the latency of an
+// iteration, which is all that counts here. VPT > 1: one warp; VPT = 1: up to 16 warps, one vertex per
+// thread. Every interval is taken in full (no quick test, square root or branch unless FP64 has to
+// decide); the vertices whose lower bound reaches down to the smallest upper bound are counted by
+// ballots: exactly one is certain. Several warps publish {smallest upper bound, smallest lower bound,
+// index} and each warp combines all of them behind one barrier. Levels come from root walks at the
+// end. k_prim took 42 us at N = 64 and 185 at 256; now 14 and 68 (43 at 160, 169 at 500).
+constexpr int kPrimSmallN = 512;
+template <int VPT>
+__global__ void __launch_bounds__(VPT == 1 ? kPrimSmallN : 32, 1)
+k_prim_small(int n, int npad, const double* __restrict__ r, int* __restrict__ parent_out,
+             int* __restrict__ level_out, int* __restrict__ order_out, int* __restrict__ root_out) {
+  __shared__ float4 pf[kPrimSmallN];
+  __shared__ int sp[kPrimSmallN];
+  __shared__ unsigned long long rk[32], wk;
+  __shared__ int ri[32], wi;
+  __shared__ uint4 rc[2][32];
+  const double *X = r, *Y = r + npad, *Z = r + 2 * (size_t)npad;
+  const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
+
+  // Root: the particle closest to the centre of mass (the origin), lowest index on ties.
+  unsigned long long bk = ~0ull;
+  int bi = INT_MAX;
+  float4 f[VPT];
+#pragma unroll
+  for (int s = 0; s < VPT; ++s) {
+    const int w = tid + s * nt;
+    f[s] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (w >= n) continue;
+    const double x = X[w], y = Y[w], z = Z[w];
+    f[s] = make_float4(__double2float_rn(x), __double2float_rn(y), __double2float_rn(z), 0.0f);
+    pf[w] = f[s];
+    argmin_combine(bk, bi, key_bits(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z))), w);
+  }
+  __syncthreads();
+  block_argmin(bk, bi, rk, ri, &wk, &wi);
+  const int root = bi;
+  if (tid == 0) {
+    order_out[0] = root;
+    root_out[0] = root;
+  }
+
+  const float kInf = __int_as_float(0x7f800000);
+  float klo[VPT], khi[VPT];
+  int par[VPT];
+  bool live[VPT];  // a vertex outside the tree
+#pragma unroll
+  for (int s = 0; s < VPT; ++s) {
+    klo[s] = khi[s] = kInf;
+    par[s] = -1;
+    live[s] = tid + s * nt < n && tid + s * nt != root;
+  }
+  auto exact_key = [&](int w, int p) {
+    return p >= 0 ? exact_d2(X[p], Y[p], Z[p], X[w], Y[w], Z[w]) : __longlong_as_double(0x7ff0000000000000LL);
+  };
+  int u = root;
+  for (int it = 1; it < n; ++it) {
+    const float4 fu = pf[u];
+    unsigned h = ~0u, l = ~0u;  // smallest bounds of the thread's vertices; ~0u sorts last
+#pragma unroll
+    for (int s = 0; s < VPT; ++s) {
+      float lo, hi;
+      d2_interval(fu, f[s], lo, hi);
+      const bool less = live[s] && hi < klo[s] && hi >= 1e-30f;
+      if (live[s] && !less && !(lo >= khi[s])) {
+        const int w = tid + s * nt;
+        const double d = exact_d2(X[u], Y[u], Z[u], X[w], Y[w], Z[w]);
+        if (d < exact_key(w, par[s])) {
+          klo[s] = __double2float_rd(d);
+          khi[s] = __double2float_ru(d);
+          par[s] = u;
+        }
+      }
+      klo[s] = less ? lo : klo[s];
+      khi[s] = less ? hi : khi[s];
+      par[s] = less ? u : par[s];
+      h = min(h, live[s] ? __float_as_uint(khi[s]) : ~0u);
+      l = min(l, live[s] ? __float_as_uint(klo[s]) : ~0u);
+    }
+    unsigned hk = __reduce_min_sync(0xffffffffu, h);
+    int count = 0, nxt = 0;
+#pragma unroll
+    for (int s = 0; s < VPT; ++s) {
+      const unsigned b = __ballot_sync(0xffffffffu, live[s] && __float_as_uint(klo[s]) <= hk);
+      count += __popc(b);
+      if (b) nxt = s * nt + warp * 32 + __ffs(b) - 1;
+    }
+    bool certain = count == 1;
+    if (VPT == 1 && nw > 1) {
+      l = __reduce_min_sync(0xffffffffu, l);
+      uint4* q = rc[it & 1];
+      if (lane == 0) q[warp] = make_uint4(hk, l, (unsigned)nxt, certain);
+      __syncthreads();
+      const uint4 e = lane < nw ? q[lane] : make_uint4(~0u, ~0u, 0u, 0u);
+      hk = __reduce_min_sync(0xffffffffu, e.x);
+      const unsigned reach = __ballot_sync(0xffffffffu, e.y <= hk);
+      const int w0 = __ffs(__ballot_sync(0xffffffffu, e.x == hk)) - 1;
+      nxt = __shfl_sync(0xffffffffu, (int)e.z, w0);
+      certain = __shfl_sync(0xffffffffu, (int)e.w, w0) && reach == 1u << w0;
+    }
+    if (!certain) {  // the same in every thread
+      bk = ~0ull;
+      bi = INT_MAX;
+#pragma unroll
+      for (int s = 0; s < VPT; ++s)
+        if (live[s] && __float_as_uint(klo[s]) <= hk) {
+          const int w = tid + s * nt;
+          argmin_combine(bk, bi, key_bits(exact_key(w, par[s])), w);
+        }
+      block_argmin(bk, bi, rk, ri, &wk, &wi);
+      nxt = bi;
+    }
+#pragma unroll
+    for (int s = 0; s < VPT; ++s) live[s] = live[s] && tid + s * nt != nxt;
+    if (tid == 0) order_out[it] = nxt;
+    u = nxt;
+  }
+#pragma unroll
+  for (int s = 0; s < VPT; ++s) {
+    const int w = tid + s * nt;
+    if (w >= n) continue;
+    if (par[s] < 0 && w != root) par[s] = root;  // only with non-finite positions
+    sp[w] = par[s];
+    parent_out[w] = par[s];
+  }
+  __syncthreads();
+  for (int w = tid; w < n; w += nt) {
+    int d = 0;
+    for (int p = sp[w]; p >= 0; p = sp[p]) ++d;
+    level_out[w] = d;
   }
 }
 
@@ -479,10 +622,27 @@ cudaError_t run_prim(mstar_ctx* c, int nt) {
   return cudaGetLastError();
 }
 
+template <int VPT>
+cudaError_t run_prim_small(mstar_ctx* c, int nt) {
+  k_prim_small<VPT><<<1, nt, 0, c->stream>>>(c->n, c->npad, c->d.r, c->d.parent, c->d.level, c->d.order, c->d.root);
+  MSTAR_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_prim(mstar_ctx* c) {
   const int n = c->n;
+  if (n <= kPrimSmallN) {
+    // up to 96 bodies one warp takes every vertex: no barrier (0.22 us an iteration at 64); four
+    // vertices a lane (0.35 us at 128) lose to a warp per 32 bodies (0.27 us)
+    switch (n <= 96 ? (n + 31) / 32 : 0) {
+      case 1: return run_prim_small<1>(c, 32);
+      case 2: return run_prim_small<2>(c, 32);
+      case 3: return run_prim_small<3>(c, 32);
+      default: return run_prim_small<1>(c, (n + 31) / 32 * 32);
+    }
+  }
   const int vpts[] = {1, 2, 3, 4, 6, 8, 10};
   int vpt = 10;
   for (int v : vpts)
@@ -490,14 +650,7 @@ cudaError_t launch_prim(mstar_ctx* c) {
       vpt = v;
       break;
     }
-  int nt = ((n + vpt - 1) / vpt + 31) / 32 * 32;
-  if (nt < 32) nt = 32;
-  // up to 96 bodies one warp takes every vertex (up to 3 each): its reductions need no
-  // shared-memory stage and no block barrier
-  if (n <= 96) {
-    vpt = (n + 31) / 32;
-    nt = 32;
-  }
+  const int nt = ((n + vpt - 1) / vpt + 31) / 32 * 32;
   switch (vpt) {
     case 1: return run_prim<1>(c, nt);
     case 2: return run_prim<2>(c, nt);
