@@ -30,6 +30,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "pairtile.cuh"
 
 namespace mstar {
 namespace {
@@ -257,11 +258,26 @@ struct NearWalk {
   }
 };
 
-// One 32-block of partners and their accumulators, per warp.
+// One 32-block of partners and their accumulators, per warp: SubTile's arrays, and what the sweep
+// of a narrow last block needs. Arrays that are never needed together share their place (a warp's
+// barrier between): positions and integer sums, fixed-point positions and tree indices, float copies
+// and masses.
 struct WarpShared {
-  double x[32], y[32], z[32], mm[32], ax[32], ay[32], az[32];
+  union {
+    struct { double x[32], y[32], z[32]; };
+    struct { long long bx[32], by[32], bz[32]; };
+  };
+  union {
+    struct { long long fx[32], fy[32], fz[32]; };
+    struct { int p[32], g[32]; };
+  };
+  union {
+    float4 f[32];
+    double mm[32];
+  };
+  double ax[32], ay[32], az[32];
   unsigned long long ms[32];
-  int me[32], p[32], g[32];
+  int me[32], cj[32];
 };
 
 // Pair loop of one system by one group: accelerations (3-vectors, times G) into a0 (the
@@ -287,61 +303,94 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
   for (int I = 0; I < nb; ++I) {
     for (int J = I; J < nb; ++J, ++q) {
       if ((q & (G - 1)) != gi.w) continue;
-      const int i = I * 32 + lane;
-      const bool ipad = i >= n;
+      const int i = I * 32 + lane, jb = J * 32 + lane;
+      const bool ipad = i >= n, jpad = jb >= n, self = I == J;
       const double xi = ipad ? 0.0 : r[3 * i], yi = ipad ? 0.0 : r[3 * i + 1], zi = ipad ? 0.0 : r[3 * i + 2];
-      const MassSplit msi = mass_split(ipad ? 1.0 : m[i]);
-      const double mi = ipad ? 0.0 : m[i];
+      const double xj = jpad ? 0.0 : r[3 * jb], yj = jpad ? 0.0 : r[3 * jb + 1], zj = jpad ? 0.0 : r[3 * jb + 2];
+      const double mi = ipad ? 0.0 : m[i], mjb = jpad ? 0.0 : m[jb];
       const int pi = ipad ? -3 : parent[i], gpi = ipad ? -3 : gp[i];
+      const int pjb = jpad ? -3 : parent[jb], gjb = jpad ? -3 : gp[jb];
       double axi = 0.0, ayi = 0.0, azi = 0.0, ui = 0.0;
-      const int jb = J * 32 + lane;
-      const bool jpad = jb >= n;
-      sh.x[lane] = jpad ? 0.0 : r[3 * jb];
-      sh.y[lane] = jpad ? 0.0 : r[3 * jb + 1];
-      sh.z[lane] = jpad ? 0.0 : r[3 * jb + 2];
-      sh.mm[lane] = jpad ? 0.0 : m[jb];
-      const MassSplit ms = mass_split(jpad ? 1.0 : m[jb]);
-      sh.ms[lane] = ms.m;
-      sh.me[lane] = ms.e;
-      sh.p[lane] = jpad ? -3 : parent[jb];
-      sh.g[lane] = jpad ? -3 : gp[jb];
+      sh.x[lane] = xj;
+      sh.y[lane] = yj;
+      sh.z[lane] = zj;
       sh.ax[lane] = 0.0;
       sh.ay[lane] = 0.0;
       sh.az[lane] = 0.0;
-      __syncwarp();
       // A partner block with t < 32 bodies (the last one) is swept at width Wb = the power of
       // two >= t: lane l pairs with slot (l + k) mod Wb, Wb steps (Wb/2 + 1 on the diagonal),
       // and the 32 / Wb lane groups keep separate partner accumulators (added below in group
       // order), so that no two lanes update the same accumulator at a step.
-      const bool self = (I == J);
       const int tail = n - J * 32;
       const int Wb = tail >= 32 ? 32 : (1 << (32 - __clz(tail - 1)));
-      const int cb = lane & ~(Wb - 1);
-      const int kbeg = self ? 1 : 0, kend = self ? Wb / 2 + 1 : Wb;
-      for (int k = kbeg; k < kend; ++k) {
-        const int jl = (lane + k) & (Wb - 1);
-        const int ja = cb + jl;
-        const int j = J * 32 + jl;
-        bool masked = ipad | (j >= n) | (self & (k == Wb / 2) & ((lane & (Wb - 1)) >= Wb / 2));
-        const int pj = sh.p[jl], gj = sh.g[jl];
-        masked |= nd1 & ((pi == j) | (pj == i));
-        masked |= nd2 & ((gpi == j) | (gj == i) | (pi == pj));
-        double dx = sh.x[jl] - xi, dy = sh.y[jl] - yi, dz = sh.z[jl] - zi;
-        asm volatile("" : "+d"(dx), "+d"(dy), "+d"(dz));
-        double rinv, sj, si;
-        if (!masked) {
-          pair_scalars_int(dx, dy, dz, MassSplit{sh.ms[jl], sh.me[jl]}, msi, rinv, sj, si);
-        } else {
-          rinv = sj = si = 0.0;
-        }
-        axi = fma(sj, dx, axi);
-        ayi = fma(sj, dy, ayi);
-        azi = fma(sj, dz, azi);
-        ui = fma(sh.mm[jl], rinv, ui);
-        sh.ax[ja] = fma(si, dx, sh.ax[ja]);
-        sh.ay[ja] = fma(si, dy, sh.ay[ja]);
-        sh.az[ja] = fma(si, dz, sh.az[ja]);
+      if (Wb == 32) {  // the arithmetic of the large systems' pair loop
+        const double pi3[3] = {xi, yi, zi}, pj3[3] = {xj, yj, zj};
+        const double m0 = m[I * 32];
+        bool eq;
+        const FixWindow fw = tile_window<1>(pi3, pj3, mi, mjb, ipad, jpad, m0, nullptr, &eq);
+        sh.fx[lane] = fix_of(xj, fw.u);
+        sh.fy[lane] = fix_of(yj, fw.u);
+        sh.fz[lane] = fix_of(zj, fw.u);
+        sh.f[lane] = make_float4(__double2float_rn(xj), __double2float_rn(yj), __double2float_rn(zj),
+                                 __double2float_rn(mjb));
+        const MassSplit ms = fix_mass(mjb);
+        sh.ms[lane] = ms.m;
+        sh.me[lane] = ms.e;
+        const int k0 = self ? 1 : 0, k1 = self ? 17 : 32;
+        unsigned mw = mask_word(nullptr, ipad, tail, self, lane);
+        if (nd1)
+          for (int k = k0; k < k1; ++k) {
+            const int q = (lane + k) & 31, j = J * 32 + q;
+            const int pj = __shfl_sync(0xffffffffu, pjb, q), gj = __shfl_sync(0xffffffffu, gjb, q);
+            const bool near = (pi == j) | (pj == i) | (nd2 & ((gpi == j) | (gj == i) | (pi == pj)));
+            mw |= near ? 1u << k : 0u;
+          }
+        TileBody body;
+        body.set(xi, yi, zi, mi, fw);
         __syncwarp();
+        const SubTile t{sh.x,  sh.y,  sh.z,  sh.fx, sh.fy, sh.fz, sh.ms, sh.me, sh.f,
+                        nullptr, sh.ax, sh.ay, sh.az, sh.bx, sh.by, sh.bz, sh.cj};
+        subtile_pairs<false>(body, t, fw, eq, m0, mw, k0, k1, lane);
+        axi = body.ax;
+        ayi = body.ay;
+        azi = body.az;
+        ui = body.u_sum();
+      } else {
+        const MassSplit msi = mass_split(ipad ? 1.0 : mi);
+        const MassSplit ms = mass_split(jpad ? 1.0 : mjb);
+        sh.mm[lane] = mjb;
+        sh.ms[lane] = ms.m;
+        sh.me[lane] = ms.e;
+        sh.p[lane] = pjb;
+        sh.g[lane] = gjb;
+        __syncwarp();
+        const int cb = lane & ~(Wb - 1);
+        const int kbeg = self ? 1 : 0, kend = self ? Wb / 2 + 1 : Wb;
+        for (int k = kbeg; k < kend; ++k) {
+          const int jl = (lane + k) & (Wb - 1);
+          const int ja = cb + jl;
+          const int j = J * 32 + jl;
+          bool masked = ipad | (j >= n) | (self & (k == Wb / 2) & ((lane & (Wb - 1)) >= Wb / 2));
+          const int pj = sh.p[jl], gj = sh.g[jl];
+          masked |= nd1 & ((pi == j) | (pj == i));
+          masked |= nd2 & ((gpi == j) | (gj == i) | (pi == pj));
+          double dx = sh.x[jl] - xi, dy = sh.y[jl] - yi, dz = sh.z[jl] - zi;
+          asm volatile("" : "+d"(dx), "+d"(dy), "+d"(dz));
+          double rinv, sj, si;
+          if (!masked) {
+            pair_scalars_int(dx, dy, dz, MassSplit{sh.ms[jl], sh.me[jl]}, msi, rinv, sj, si);
+          } else {
+            rinv = sj = si = 0.0;
+          }
+          axi = fma(sj, dx, axi);
+          ayi = fma(sj, dy, ayi);
+          azi = fma(sj, dz, azi);
+          ui = fma(sh.mm[jl], rinv, ui);
+          sh.ax[ja] = fma(si, dx, sh.ax[ja]);
+          sh.ay[ja] = fma(si, dy, sh.ay[ja]);
+          sh.az[ja] = fma(si, dz, sh.az[ja]);
+          __syncwarp();
+        }
       }
       // body jb and body i of this item are only ever touched by this lane of this warp
       if (!jpad) {  // partner sums were kept with the opposite sign
@@ -819,7 +868,8 @@ __device__ void attempt_finish(const SysView& V, SysScalars* S, const BatchParam
 // finishes it.
 template <int G>
 __global__ void __launch_bounds__(128 * G) k_batched_step(MSTAR_BSTEP_ARGS) {
-  __shared__ WarpShared wsh[4 * G];
+  extern __shared__ __align__(16) unsigned char wsh_mem[];  // 4 G WarpShared
+  WarpShared* wsh = reinterpret_cast<WarpShared*>(wsh_mem);
   __shared__ unsigned long long rk[4 * G];
   __shared__ int ri[4 * G];
   __shared__ int s_cnt[kBMaxN + 1];
@@ -848,7 +898,8 @@ __global__ void __launch_bounds__(128 * G) k_batched_step(MSTAR_BSTEP_ARGS) {
 // order[i]) and the finish (one CTA per system).
 template <int G>
 __global__ void __launch_bounds__(128 * G) k_bsplit_begin(MSTAR_BSTEP_ARGS) {
-  __shared__ WarpShared wsh[4 * G];
+  extern __shared__ __align__(16) unsigned char wsh_mem[];  // 4 G WarpShared
+  WarpShared* wsh = reinterpret_cast<WarpShared*>(wsh_mem);
   __shared__ unsigned long long rk[4 * G];
   __shared__ int ri[4 * G];
   __shared__ int s_cnt[kBMaxN + 1];
@@ -864,7 +915,8 @@ __global__ void __launch_bounds__(128 * G) k_bsplit_begin(MSTAR_BSTEP_ARGS) {
 
 template <int G>
 __global__ void __launch_bounds__(32 * G) k_bsplit_div(MSTAR_BSTEP_ARGS) {
-  __shared__ WarpShared wsh[G];
+  extern __shared__ __align__(16) unsigned char wsh_mem[];  // G WarpShared
+  WarpShared* wsh = reinterpret_cast<WarpShared*>(wsh_mem);
   __shared__ double s_gred[kGroups][kMaxG][3];
   const int item = (int)(blockIdx.x >> 2), g = (int)(blockIdx.x & 3);
   if (item >= count) return;
@@ -1472,13 +1524,15 @@ int apply_schedule(mstar_batch* b, const int* sched) {
   bool ok = true;
   int nodes = 0;
   static const int node_order[kNodeKinds] = {7, 2, 6, 1, 5, 0, 4, 3, 8};  // widest groups first
-  auto add_node = [&](void* func, dim3 grid, dim3 block, void** args, const cudaGraphNode_t* dep, int prio,
-                      cudaGraphNode_t* node) {
+  auto add_node = [&](void* func, dim3 grid, dim3 block, size_t smem, void** args, const cudaGraphNode_t* dep,
+                      int prio, cudaGraphNode_t* node) {
+    if (smem && cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return false;
     cudaKernelNodeParams kp{};
     kp.func = func;
     kp.gridDim = grid;
     kp.blockDim = block;
-    kp.sharedMemBytes = 0;
+    kp.sharedMemBytes = (unsigned)smem;
     kp.kernelParams = args;
     if (cudaGraphAddKernelNode(node, graph, dep, dep ? 1 : 0, &kp) != cudaSuccess) return false;
     cudaLaunchAttributeValue pv{};
@@ -1502,11 +1556,11 @@ int apply_schedule(mstar_batch* b, const int* sched) {
       const int per = mstar::kSegThreads / (4 * wd);
       void* f = qi == 8 ? (void*)mstar::k_batched_seg<4>
                         : (qi == 3 ? (void*)mstar::k_batched_seg<8> : (void*)mstar::k_batched_seg<16>);
-      ok = add_node(f, dim3((cnt + per - 1) / per), dim3(mstar::kSegThreads), args, nullptr, lo_prio, &n0);
+      ok = add_node(f, dim3((cnt + per - 1) / per), dim3(mstar::kSegThreads), 0, args, nullptr, lo_prio, &n0);
     } else if (qi < 3) {
       void* f = G == 1 ? (void*)mstar::k_batched_step<1> : (G == 2 ? (void*)mstar::k_batched_step<2>
                                                                    : (void*)mstar::k_batched_step<4>);
-      ok = add_node(f, dim3(cnt), dim3(128 * G), args, nullptr, prio, &n0);
+      ok = add_node(f, dim3(cnt), dim3(128 * G), 4 * G * sizeof(mstar::WarpShared), args, nullptr, prio, &n0);
     } else {
       void* fb = G == 1 ? (void*)mstar::k_bsplit_begin<1> : (G == 2 ? (void*)mstar::k_bsplit_begin<2>
                                                                     : (void*)mstar::k_bsplit_begin<4>);
@@ -1514,9 +1568,9 @@ int apply_schedule(mstar_batch* b, const int* sched) {
                                                                   : (void*)mstar::k_bsplit_div<4>);
       void* ff = G == 1 ? (void*)mstar::k_bsplit_finish<1> : (G == 2 ? (void*)mstar::k_bsplit_finish<2>
                                                                      : (void*)mstar::k_bsplit_finish<4>);
-      ok = add_node(fb, dim3(cnt), dim3(128 * G), args, nullptr, prio, &n0) &&
-           add_node(fd, dim3(4 * cnt), dim3(32 * G), args, &n0, prio, &n1) &&
-           add_node(ff, dim3(cnt), dim3(128 * G), args, &n1, prio, &n2);
+      ok = add_node(fb, dim3(cnt), dim3(128 * G), 4 * G * sizeof(mstar::WarpShared), args, nullptr, prio, &n0) &&
+           add_node(fd, dim3(4 * cnt), dim3(32 * G), G * sizeof(mstar::WarpShared), args, &n0, prio, &n1) &&
+           add_node(ff, dim3(cnt), dim3(128 * G), 0, args, &n1, prio, &n2);
     }
   }
   cudaGetLastError();
