@@ -348,8 +348,7 @@ int issue_attempt(mstar_ctx* c) {
       CK(save(tr->SC + tau * nsc, c->d.sc, nsc));
     }
     if (lo2 < K)
-      CK(launch_rebuild(c, c->d.sX + lo2 * st, c->d.sr + lo2 * st, st, K - lo2, 0, nullptr,
-                        c->d.comblk + (size_t)lo2 * c->nblk * 3));
+      CK(launch_rebuild(c, c->d.sX + lo2 * st, c->d.sr + lo2 * st, st, K - lo2, 0, nullptr, nullptr));
   }
   if ((rc = join_start_eval(c))) return rc;
   CK(launch_extrapolate(c));
@@ -387,8 +386,7 @@ int issue_attempt_branched(mstar_ctx* c) {
                            c->d.comblk + (size_t)k * c->nblk * 3);
       if (e == cudaSuccess) e = launch_drift(c, k, k + 1, tau);
       if (e == cudaSuccess && pos == k)
-        e = launch_rebuild(c, c->d.sX + k * st, c->d.sr + k * st, st, 1, 0, nullptr,
-                           c->d.comblk + (size_t)k * c->nblk * 3);
+        e = launch_rebuild(c, c->d.sX + k * st, c->d.sr + k * st, st, 1, 0, nullptr, nullptr);
     }
     if (e == cudaSuccess) e = cudaEventRecord(c->br_join[k], c->stream);
   }

@@ -187,7 +187,8 @@ __device__ __forceinline__ void component_block_sums(double x, double* scratch, 
 // + ... up to the root (root: 0), plus block sums of m w for the centre of mass. A CTA takes
 // kBlock bodies with one thread per component, so the three walks of a body run side by side
 // (each adds in the same order as one thread walking all three); beside pair launches of other
-// divisions, which keep the FP64 pipe busy, the walks' share of the pipe grows with their warps.
+// divisions the walks' share of an SM grows with their warps. comblk null: no block sums (positions
+// for pair sums alone, which stay relative to the root).
 __global__ void __launch_bounds__(kBlock * kRebuildComps)
 k_rebuild(int n, int npad, size_t stride, const int* __restrict__ parent, const int* __restrict__ bylev,
           const double* __restrict__ Wb, double* __restrict__ wb, const double* __restrict__ m,
@@ -205,6 +206,7 @@ k_rebuild(int n, int npad, size_t stride, const int* __restrict__ parent, const 
     for (int u = v; parent[u] >= 0; u = parent[u]) s = __dadd_rn(s, W[u]);
     wv[v] = s;
   }
+  if (!comblk) return;
   const double mv = v < n ? m[v] : 0.0;
   component_block_sums(__dmul_rn(mv, s), scratch, comblk + ((size_t)slot * nblk + blockIdx.x) * 3);
 }
@@ -247,118 +249,134 @@ k_rebuild_staged(int n, int npad, size_t stride, const int* __restrict__ parent,
     for (int u = v; sP[u] >= 0; u = sP[u]) s = __dadd_rn(s, sWc[u]);
     wv[v] = s;
   }
+  if (!comblk) return;
   const double mv = v < n ? m[v] : 0.0;
   component_block_sums(__dmul_rn(mv, s), scratch, comblk + ((size_t)slot * nblk + blockIdx.x) * 3);
 }
 
-// Sum over the CTA, returned to every thread (block_sum leaves it in thread 0).
-__device__ __forceinline__ double cta_sum(double x, double* scratch, double* out) {
-  const double b = block_sum(x, scratch);
-  if (threadIdx.x == 0) *out = b;
-  __syncthreads();
-  return *out;
-}
-
-// The Cartesian vectors of the edge vectors in sW (3 planes, shared) by path sums over the
-// staged parents sP, shifted to the centre-of-mass frame and written to w_out; returns
-// m w^2 of the thread's body (0 for none). One body per thread (blockDim >= n), in tree-level
-// order; every thread of the CTA calls it (it holds barriers).
-__device__ __forceinline__ double rebuild_cta(int n, int npad, double Mtot, const double* __restrict__ m,
-                                              const int* sP, const int* __restrict__ bylev, const double* sW,
-                                              double* w_out, double* scratch, double* s_bc) {
-  const int tid = threadIdx.x;
-  const int v = tid < n ? bylev[tid] : n;
-  double q[3] = {0.0, 0.0, 0.0};
-  if (v < n)
-    for (int u = v; sP[u] >= 0; u = sP[u]) {
-      q[0] = __dadd_rn(q[0], sW[u]);
-      q[1] = __dadd_rn(q[1], sW[npad + u]);
-      q[2] = __dadd_rn(q[2], sW[2 * (size_t)npad + u]);
-    }
-  const double mv = v < n ? m[v] : 0.0;
-  double com[3];
-  for (int c = 0; c < 3; ++c) com[c] = cta_sum(__dmul_rn(mv, q[c]), scratch, &s_bc[1 + c]);
-  double t2 = 0.0;
-  if (v < n) {
-    for (int c = 0; c < 3; ++c) {
-      q[c] = __dsub_rn(q[c], com[c] / Mtot);
-      w_out[(size_t)c * npad + v] = q[c];
-    }
-    t2 = __dmul_rn(mv, __dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])), __dmul_rn(q[2], q[2])));
-  }
-  return t2;
-}
-
-// One substep level tau of division `slot` on the CTA: the kick K(delta) of k_kick with the
-// accelerations a (3 planes) and force function U, the velocities rebuilt by path sums and
-// shifted to the centre-of-mass frame with their kinetic energy (k_rebuild, k_shift), the
-// drift of k_drift, and, when `pos` (the division kicks again), the positions rebuilt and
-// shifted into r_out. Every thread of the CTA calls it; sW is 3 npad doubles of scratch.
-__device__ __forceinline__ void level_body(int n, int npad, int slot, bool pos, double H, double B, double Mtot,
-                                           int tau, double U, const double* a, const double* __restrict__ m,
-                                           const int* sP, const int* __restrict__ bylev, double* V, double* X,
-                                           double* sW, double* v_out, double* r_out, double* scratch, double* s_bc,
-                                           double* __restrict__ sc) {
-  const int tid = threadIdx.x;
-  // K(delta): V_w += (delta / U) (a_w - a_parent(w))
-  const double fk = (H / (double)(2 * (slot + 1))) / U;
-  for (int w = tid; w < npad; w += blockDim.x) {
-    const int p = sP[w];
-    for (int c = 0; c < 3; ++c) {
-      const size_t o = (size_t)c * npad + w;
-      double x = V[o];
-      if (p >= 0) x = madd(x, fk, __dsub_rn(a[o], a[(size_t)c * npad + p]));
-      V[o] = x;
-      sW[o] = x;
-    }
-  }
-  if (tid == 0) sc[slot * kScal + SC_U] = U;
-  __syncthreads();
-  const double T = 0.5 * cta_sum(rebuild_cta(n, npad, Mtot, m, sP, bylev, sW, v_out, scratch, s_bc), scratch,
-                                 &s_bc[4]);
-  // D(h): X += f V, t += f with f = h / (T + B); h = delta, or delta/2 for the last drift
-  const int nk = 2 * (slot + 1);
-  const double delta = H / (double)nk;
-  const double h = (tau == nk) ? 0.5 * delta : delta;
-  const double fd = h / (T + B);
-  for (int w = tid; w < npad; w += blockDim.x)
-    for (int c = 0; c < 3; ++c) {
-      const size_t o = (size_t)c * npad + w;
-      const double x = madd(X[o], fd, V[o]);
-      X[o] = x;
-      sW[o] = x;
-    }
-  if (tid == 0) {
-    sc[slot * kScal + SC_T_PHYS] += fd;
-    sc[slot * kScal + SC_T_KIN] = T;
-  }
-  __syncthreads();
-  if (pos) rebuild_cta(n, npad, Mtot, m, sP, bylev, sW, r_out, scratch, s_bc);
-}
-
-// One substep level of every active division of a system that one CTA holds (npad <= 1024,
-// one body per thread; the step uses it up to kLevelCtaMax): level_body with the
-// accelerations and force-function partials of the pair kernels - six launches of the
-// multi-CTA path in one, with the CTA's barriers in place of the kernel boundaries. The
-// edge vectors are staged in shared memory for the walks. The operations are those of the
-// multi-CTA kernels; the centre-of-mass and kinetic sums are CTA-wide instead of per 64-body
-// block, so they round in another order.
-__global__ void __launch_bounds__(1024)
+// One substep level of every active division of a system that one CTA holds (npad <= kLevelCtaMax,
+// one body per thread), with the accelerations and force-function partials of the pair kernels: the
+// kick of k_kick, the velocities rebuilt by path sums and shifted to the centre-of-mass frame with
+// their kinetic energy (k_rebuild, k_shift), the drift of k_drift and, when the division kicks again,
+// the positions by path sums. Six launches of the multi-CTA path in one, with the CTA's barriers in
+// place of the kernel boundaries. The operations are those of the multi-CTA kernels; the
+// centre-of-mass and kinetic sums are CTA-wide instead of per 64-body block, so they round in another
+// order.
+//
+// Bound by the SM's FP64 pipe (an instruction of a warp holds it 16 cycles; a division is some ten)
+// and the chain of sums. So whatever all bodies share is computed once: each quotient by one thread,
+// and the sums by a warp per component over products left in shared memory. 23.8 us a level at
+// N = 256 when every warp divided for itself and positions were shifted too; now 16.8.
+__global__ void __launch_bounds__(kLevelCtaMax)
 k_level_cta(int n, int npad, int slot_lo, int pos_lo, const double* __restrict__ par, double B, double Mtot,
             int tau, const double* __restrict__ m, const int* __restrict__ parent, const int* __restrict__ bylev,
             const double* __restrict__ sa, double* __restrict__ sV, double* __restrict__ sv, double* __restrict__ sX,
             double* __restrict__ sr, const double* __restrict__ Ublk, int nblk, double* __restrict__ sc) {
-  extern __shared__ __align__(16) double lvl_sh[];  // 3 npad staged edge vectors, then npad parents
+  extern __shared__ __align__(16) double lvl_sh[];  // 3 npad edge vectors, 3 npad products, npad parents
   double* sW = lvl_sh;
-  int* sP = reinterpret_cast<int*>(lvl_sh + 3 * (size_t)npad);
-  __shared__ double scratch[32];
-  __shared__ double s_bc[8];
+  double* sM = sW + 3 * (size_t)npad;
+  int* sP = reinterpret_cast<int*>(sM + 3 * (size_t)npad);
+  __shared__ double s_com[3], s_U, s_fk, s_T, s_fd;
   const int slot = slot_lo + blockIdx.x;
   const size_t st = (size_t)3 * npad;
-  for (int u = threadIdx.x; u < npad; u += blockDim.x) sP[u] = u < n ? parent[u] : -1;
-  sum_partials(Ublk + (size_t)slot * nblk, nblk, 1, &s_bc[0]);  // ends with a barrier
-  level_body(n, npad, slot, slot >= pos_lo, par[0], B, Mtot, tau, s_bc[0], sa + slot * st, m, sP, bylev,
-             sV + slot * st, sX + slot * st, sW, sv + slot * st, sr + slot * st, scratch, s_bc, sc);
+  const int w = threadIdx.x, warp = w >> 5, lane = w & 31;  // blockDim.x == npad
+  double *V = sV + slot * st, *X = sX + slot * st;
+  const double* a = sa + slot * st;
+  const int p = w < n ? parent[w] : -1, v = w < n ? bylev[w] : n;
+  const double mv = v < n ? m[v] : 0.0;
+  double vw[3], xw[3], da[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const size_t o = (size_t)c * npad;
+    vw[c] = V[o + w];
+    xw[c] = X[o + w];
+    da[c] = p >= 0 ? __dsub_rn(a[o + w], a[o + p]) : 0.0;
+  }
+  sP[w] = p;
+  const int nk = 2 * (slot + 1);
+  const double delta = par[0] / (double)nk;
+  // sum over the products in sM[0 .. npad) by one warp, in lane 0
+  auto plane_sum = [&](const double* q) {
+    double s = 0.0;
+    for (int u = lane; u < npad; u += 32) s += q[u];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
+  };
+  auto path_sum = [&](double (&q)[3]) {
+    q[0] = q[1] = q[2] = 0.0;
+    if (v < n)
+      for (int u = v; sP[u] >= 0; u = sP[u])
+        for (int c = 0; c < 3; ++c) q[c] = __dadd_rn(q[c], sW[c * npad + u]);
+  };
+  // K(delta): V_w += (delta / U) (a_w - a_parent(w))
+  if (warp == 0) {
+    double U = 0.0;
+    for (int b = lane; b < nblk; b += 32) U += Ublk[(size_t)slot * nblk + b];
+    for (int o = 16; o > 0; o >>= 1) U += __shfl_down_sync(0xffffffffu, U, o);
+    if (lane == 0) {
+      s_U = U;
+      s_fk = delta / U;
+    }
+  }
+  __syncthreads();
+  const double fk = s_fk;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const size_t o = (size_t)c * npad + w;
+    if (p >= 0) vw[c] = madd(vw[c], fk, da[c]);
+    V[o] = vw[c];
+    sW[o] = vw[c];
+  }
+  __syncthreads();
+  // velocities, their centre of mass and kinetic energy
+  double q[3];
+  path_sum(q);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) sM[c * npad + w] = __dmul_rn(mv, q[c]);
+  __syncthreads();
+  for (int c = warp; c < 3; c += (int)(blockDim.x >> 5)) {
+    const double s = plane_sum(sM + c * npad);
+    if (lane == 0) s_com[c] = s / Mtot;
+  }
+  __syncthreads();
+  double t2 = 0.0;
+  if (v < n) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      q[c] = __dsub_rn(q[c], s_com[c]);
+      sv[slot * st + (size_t)c * npad + v] = q[c];
+    }
+    t2 = __dmul_rn(mv, __dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])), __dmul_rn(q[2], q[2])));
+  }
+  sM[w] = t2;
+  __syncthreads();
+  // D(h): X += f V, t += f with f = h / (T + B); h = delta, or delta/2 for the last drift
+  if (warp == 0) {
+    const double T = 0.5 * plane_sum(sM);
+    if (lane == 0) {
+      s_T = T;
+      s_fd = ((tau == nk) ? 0.5 * delta : delta) / (T + B);
+    }
+  }
+  __syncthreads();
+  const double fd = s_fd;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const size_t o = (size_t)c * npad + w;
+    xw[c] = madd(xw[c], fd, vw[c]);
+    X[o] = xw[c];
+    sW[o] = xw[c];
+  }
+  if (w == 0) {
+    sc[slot * kScal + SC_U] = s_U;
+    sc[slot * kScal + SC_T_PHYS] += fd;
+    sc[slot * kScal + SC_T_KIN] = s_T;
+  }
+  if (slot < pos_lo) return;
+  __syncthreads();
+  path_sum(q);
+  if (v < n)
+    for (int c = 0; c < 3; ++c) sr[slot * st + (size_t)c * npad + v] = q[c];
 }
 
 // One substep level of a division on a thread-block cluster of C CTAs, for systems too large for
@@ -416,15 +434,16 @@ __device__ __forceinline__ void cluster_walks(int n, int npad, int nblk, int ran
 }
 
 // The centre of mass from the blocks' partials (warp c sums component c in sum_partials' order)
-// into s_com[0..2]; holds a barrier.
-__device__ __forceinline__ void cluster_com(int nblk, const double* sCom, double* s_com) {
+// into s_com[0..2]; holds a barrier. The quotients here and below are formed by one thread each:
+// a division is some ten FP64 instructions, which every warp of the CTA would queue for.
+__device__ __forceinline__ void cluster_com(int nblk, double Mtot, const double* sCom, double* s_com) {
   const int tid = threadIdx.x;
   if (tid < 96) {
     const int c = tid >> 5, lane = tid & 31;
     double s = 0.0;
     for (int bb = lane; bb < nblk; bb += 32) s += sCom[bb * 3 + c];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) s_com[c] = s;
+    if (lane == 0) s_com[c] = s / Mtot;
   }
   __syncthreads();
 }
@@ -465,10 +484,13 @@ k_substep_cluster(int n, int npad, int nblk, int slot_lo, int pos_lo, int tau, c
 
   for (int u = tid; u < npad; u += blockDim.x) sP[u] = u < n ? parent[u] : -1;
   sum_partials(Ublk + (size_t)slot * nblk, nblk, 1, &s_sc[0]);  // ends with a barrier
-  const double U = s_sc[0];
+  if (tid == 0) {
+    s_sc[1] = (H / (double)(2 * (slot + 1))) / s_sc[0];
+    if (rank == 0) sc[slot * kScal + SC_U] = s_sc[0];
+  }
   cl.sync();  // every CTA of the cluster runs before any writes into its shared memory
   // K(delta), as k_kick: V_w += (delta / U) (a_w - a_parent(w))
-  const double fk = (H / (double)(2 * (slot + 1))) / U;
+  const double fk = s_sc[1];
   for (int it = 0; it < passes; ++it) {
     const int blk = (it * C + rank) * G + g;
     const int w = blk * kBlock + b;
@@ -486,12 +508,11 @@ k_substep_cluster(int n, int npad, int nblk, int slot_lo, int pos_lo, int tau, c
       for (int r = 0; r < C; ++r) cl.map_shared_rank(sW, r)[o] = x;
     }
   }
-  if (rank == 0 && tid == 0) sc[slot * kScal + SC_U] = U;
   cl.sync();
   // velocity rebuild (k_rebuild), then the shift and the kinetic partials (k_shift)
   cluster_walks<C>(n, npad, nblk, rank, G, g, comp, b, bylev, m, sP, sW, sQ, sCom, scr);
   cl.sync();
-  cluster_com(nblk, sCom, &s_sc[1]);
+  cluster_com(nblk, Mtot, sCom, &s_sc[1]);
   double* vout = sv + slot * st;
   for (int it = 0; it < passes; ++it) {
     const int blk = (it * C + rank) * G + g;
@@ -500,7 +521,7 @@ k_substep_cluster(int n, int npad, int nblk, int slot_lo, int pos_lo, int tau, c
     double q = 0.0;
     if (own) {
       const size_t o = (size_t)comp * npad + w;
-      q = __dsub_rn(sQ[o], s_sc[1 + comp] / Mtot);
+      q = __dsub_rn(sQ[o], s_sc[1 + comp]);
       vout[o] = q;
     }
     sq3[g][comp][b] = q;
@@ -529,14 +550,21 @@ k_substep_cluster(int n, int npad, int nblk, int slot_lo, int pos_lo, int tau, c
     double s = 0.0;
     for (int bb = tid; bb < nblk; bb += 32) s += sT[bb];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (tid == 0) s_sc[0] = s;
+    if (tid == 0) {
+      const double T = 0.5 * s;
+      const int nk = 2 * (slot + 1);
+      const double delta = H / (double)nk;
+      const double h = (tau == nk) ? 0.5 * delta : delta;
+      const double f = h / (T + B);
+      s_sc[0] = f;
+      if (rank == 0) {
+        sc[slot * kScal + SC_T_PHYS] += f;
+        sc[slot * kScal + SC_T_KIN] = T;
+      }
+    }
   }
   __syncthreads();
-  const double T = 0.5 * s_sc[0];
-  const int nk = 2 * (slot + 1);
-  const double delta = H / (double)nk;
-  const double h = (tau == nk) ? 0.5 * delta : delta;
-  const double fd = h / (T + B);
+  const double fd = s_sc[0];
   for (int it = 0; it < passes; ++it) {
     const int blk = (it * C + rank) * G + g;
     const int w = blk * kBlock + b;
@@ -550,23 +578,19 @@ k_substep_cluster(int n, int npad, int nblk, int slot_lo, int pos_lo, int tau, c
       }
     }
   }
-  if (rank == 0 && tid == 0) {
-    sc[slot * kScal + SC_T_PHYS] += fd;
-    sc[slot * kScal + SC_T_KIN] = T;
-  }
   if (!pos) return;  // nothing of this CTA's shared memory is read by another CTA after the last barrier
   cl.sync();
-  // position rebuild and shift (k_rebuild, k_shift)
-  cluster_walks<C>(n, npad, nblk, rank, G, g, comp, b, bylev, m, sP, sW, sQ, sCom, scr);
-  cl.sync();
-  cluster_com(nblk, sCom, &s_sc[1]);
+  // positions (k_rebuild without block sums): each walk's result goes straight out
   double* rout = sr + slot * st;
+  const double* W = sW + (size_t)comp * npad;
   for (int it = 0; it < passes; ++it) {
     const int blk = (it * C + rank) * G + g;
-    const int w = blk * kBlock + b;
-    if (blk < nblk && w < n) {
-      const size_t o = (size_t)comp * npad + w;
-      rout[o] = __dsub_rn(sQ[o], s_sc[1 + comp] / Mtot);
+    const int i = blk * kBlock + b;
+    if (blk < nblk && i < n) {
+      const int v = bylev[i];
+      double s = 0.0;
+      for (int u = v; sP[u] >= 0; u = sP[u]) s = __dadd_rn(s, W[u]);
+      rout[(size_t)comp * npad + v] = s;
     }
   }
 }
@@ -674,12 +698,22 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
   double t_phys = t0 + f0, T = T0, U = 0.0;
   __syncthreads();
 
-  // Cartesian vectors of the edge vectors W (one component per task) by path sums, shifted to
-  // the centre-of-mass frame; returns the task's m v q^2 term (0 for none)
-  auto rebuild = [&](const double* W, double* out) {
+  // Cartesian vectors of the edge vectors W (one component per task) by path sums
+  auto path_sum = [&](const double* W) {
     double q = 0.0;
     if (v < n)
       for (int u = v; sP[u] >= 0; u = sP[u]) q = __dadd_rn(q, W[(size_t)c * npad + u]);
+    return q;
+  };
+  // the positions for the pair sums stay relative to the root
+  auto positions = [&]() {
+    const double q = path_sum(X);
+    if (v < n) sx[(size_t)c * npad + v] = q;
+    __syncthreads();
+  };
+  // velocities in the centre-of-mass frame; returns the task's m v q^2 term (0 for none)
+  auto velocities = [&]() {
+    double q = path_sum(V);
     if (task) {  // warp-uniform (3 npad is a multiple of 32)
       const double s = warp_sum(__dmul_rn(mv, q));
       if (lane == 0) red[warp] = s;
@@ -694,7 +728,6 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
     double t2 = 0.0;
     if (v < n) {
       q = __dsub_rn(q, s_val[c]);
-      if (out) out[(size_t)c * npad + v] = q;
       t2 = __dmul_rn(mv, __dmul_rn(q, q));
     }
     __syncthreads();  // s_val and red are free again
@@ -719,7 +752,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
     return s_val[3];
   };
 
-  rebuild(X, sx);
+  positions();
   // the pair-sum tasks: tile pairs (in tile_pair order) times S chunks of partner steps (at most
   // 8 chunks: with 4 or 16 at most, attempts at N = 64 ... 160 took 2-16 % longer), dealt out
   // over the cluster
@@ -924,7 +957,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
     __syncthreads();
     // velocities rebuilt and shifted; T = sum m v^2 / 2
     // D(h): X += f V, t += f with f = h / (T + B); h = delta, or delta/2 for the last drift
-    T = kinetic(rebuild(V, nullptr), tau);
+    T = kinetic(velocities(), tau);
     const double fd = s_val[0];
     if (task) {
       const size_t o = (size_t)c * npad + ti;
@@ -932,7 +965,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
     }
     t_phys += fd;
     __syncthreads();
-    if (tau < nk) rebuild(X, sx);
+    if (tau < nk) positions();
   }
   // the division's final state and scalars for the extrapolation (every CTA of a cluster holds
   // the same; no CTA leaves while another may still read its partials)
@@ -960,13 +993,15 @@ k_shift(int n, int npad, size_t stride, double Mtot, double* __restrict__ wb, co
   __shared__ double sc3[3];
   const int slot = blockIdx.y;
   sum_partials3(comblk + (size_t)slot * nblk * 3, nblk, sc3);
+  if (threadIdx.x < 3) sc3[threadIdx.x] = sc3[threadIdx.x] / Mtot;
+  __syncthreads();
   double* wv = wb + slot * stride;
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   double t2 = 0.0;
   if (v < n) {
     double q[3];
     for (int c = 0; c < 3; ++c) {
-      q[c] = __dsub_rn(wv[(size_t)c * npad + v], sc3[c] / Mtot);
+      q[c] = __dsub_rn(wv[(size_t)c * npad + v], sc3[c]);
       wv[(size_t)c * npad + v] = q[c];
     }
     t2 = __dmul_rn(m[v], __dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])), __dmul_rn(q[2], q[2])));
@@ -1134,7 +1169,7 @@ cudaError_t launch_init_drift(mstar_ctx* c) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t st = (size_t)3 * c->npad;
-  return launch_rebuild(c, c->d.sX, c->d.sr, st, c->K, 0, nullptr, c->d.comblk);
+  return launch_rebuild(c, c->d.sX, c->d.sr, st, c->K, 0, nullptr, nullptr);
 }
 
 cudaError_t launch_kick(mstar_ctx* c, int slot_lo, int slot_hi) {
@@ -1168,7 +1203,7 @@ cudaError_t launch_rebuild(mstar_ctx* c, const double* W, double* w, size_t stri
   }
   MSTAR_LAUNCHED(c);
   e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || !comblk_base) return e;
   k_shift<<<grid, kBlock, 0, c->stream>>>(c->n, c->npad, stride, c->Mtot, w, c->d.m, comblk_base,
                                          want_T ? Tblk_base : nullptr, c->nblk);
   MSTAR_LAUNCHED(c);
@@ -1261,7 +1296,7 @@ cudaError_t launch_division_cta(mstar_ctx* c) {
 // One substep level (kick, velocity rebuild, drift, position rebuild) of the divisions
 // [slot_lo, slot_hi) in one launch, for systems with npad <= kLevelCtaMax.
 cudaError_t launch_level_cta(mstar_ctx* c, int slot_lo, int slot_hi, int pos_lo, int tau) {
-  const size_t smem = (size_t)c->npad * (3 * sizeof(double) + sizeof(int));
+  const size_t smem = (size_t)c->npad * (6 * sizeof(double) + sizeof(int));
   k_level_cta<<<slot_hi - slot_lo, c->npad, smem, c->stream>>>(c->n, c->npad, slot_lo, pos_lo, c->d.res + 4, c->B,
                                                             c->Mtot, tau, c->d.m, c->d.parent, c->d.bylev, c->d.sa,
                                                             c->d.sV, c->d.sv, c->d.sX, c->d.sr, c->d.Ublk, c->nblk,
