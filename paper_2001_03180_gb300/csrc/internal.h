@@ -183,15 +183,15 @@ cudaError_t launch_rebuild(mstar_ctx* c, const double* W, double* w, size_t stri
                            int want_T, double* Tblk_base, double* comblk_base);
 cudaError_t prepare_rebuild(mstar_ctx* c);  // at context creation: the staged rebuild's shared memory
 // kick, velocity rebuild, drift and position rebuild of one level in one CTA per division
-// (systems with npad <= kLevelCtaMax: up to 256 bodies, where it beats the multi-CTA path by
-// launches saved; above, one SM per division binds its path sums); the divisions >= pos_lo get
-// their positions rebuilt
-constexpr int kLevelCtaMax = 256;
+// (systems with npad <= kLevelCtaMax, where one launch and no exchange beat a cluster; above, one
+// SM per division binds its path sums: attempts at N = 192, 224 and 256 take 0.56, 0.58 and 0.60 ms
+// with it, 0.55, 0.56 and 0.56 with the clusters); the divisions >= pos_lo get their positions rebuilt
+constexpr int kLevelCtaMax = 160;
 cudaError_t launch_level_cta(mstar_ctx* c, int slot_lo, int slot_hi, int pos_lo, int tau);
 // the same level of a division on a thread-block cluster (kLevelCtaMax < npad <= kSubstepClusterMax),
 // in the level-by-level schedule: bit-identical to the multi-kernel kick, rebuild, shift and drift
-// launches it replaces. Level-by-level steps of Plummer spheres with a central binary took 5-7 %
-// less time with it from 260 to 500 bodies, and 1-2 % more at 640 and 800; beside the pair loops
+// launches it replaces. Level-by-level steps of Plummer spheres with a central binary take 8-10 %
+// less time with it from 288 to 512 bodies, 3 % at 576, and 1 % more at 601, 4 % at 800; beside the pair loops
 // of other divisions (a stream per division) the clusters wait for whole SMs and slow those loops
 constexpr int kSubstepClusterMax = 576;
 cudaError_t prepare_substep_cluster(mstar_ctx* c);  // at context creation; sets sub_cluster

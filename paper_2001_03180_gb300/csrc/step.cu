@@ -266,7 +266,7 @@ k_rebuild_staged(int n, int npad, size_t stride, const int* __restrict__ parent,
 // Bound by the SM's FP64 pipe (an instruction of a warp holds it 16 cycles; a division is some ten)
 // and the chain of sums. So whatever all bodies share is computed once: each quotient by one thread,
 // and the sums by a warp per component over products left in shared memory. 23.8 us a level at
-// N = 256 when every warp divided for itself and positions were shifted too; now 16.8.
+// N = 256 when every warp divided for itself and positions were shifted too, then 16.8.
 __global__ void __launch_bounds__(kLevelCtaMax)
 k_level_cta(int n, int npad, int slot_lo, int pos_lo, const double* __restrict__ par, double B, double Mtot,
             int tau, const double* __restrict__ m, const int* __restrict__ parent, const int* __restrict__ bylev,
