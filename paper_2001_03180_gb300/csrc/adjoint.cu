@@ -212,13 +212,61 @@ k_adj_pair(int n, int npad, int slot_lo, double G, double H, const double* __res
 // The same VJP sums over every unordered pair once, in the tiling of the forward pair loop:
 // CTA (I, J), I <= J, holds tile I's bodies in registers and stages tile J's positions,
 // masses, adjoints and accumulators in shared memory; at step k of a 32-wide sub-tile lane l
-// pairs with partner (l + k) mod 32, so the lanes update distinct partner accumulators. For
-// d = r_j - r_i and w = m_i L_j - m_j L_i the pair gives
-//   u = w / r^3 - 3 d (d . w) / r^5:   mu_i += u, mu_j -= u   (M_ij = M_ji, w_ji = -w_ij)
-//   nu_i -= (L_j . d) / r^3,  nu_j += (L_i . d) / r^3,  phi_i += m_j / r,  phi_j += m_i / r,
-// about half the FP64 work of visiting each ordered pair. CTA (I, J) writes tile I's sums to
-// partial slot J and tile J's to slot I (a diagonal CTA writes both into slot I), so each
-// body receives one write per slot; the consumer adds the NT slots in order.
+// pairs with partner (l + k) mod 32, so the lanes update distinct partner accumulators. With
+// d = r_j - r_i, l = L / m and w = m_i L_j - m_j L_i = m_i m_j (l_j - l_i) the pair gives
+//   u = w / r^3 - 3 d (d . w) / r^5 = m_i m_j y / r^3,  y = (l_j - l_i) - 3 d (d . (l_j - l_i)) / r^2:
+//   mu_i += u, mu_j -= u   (M_ij = M_ji, w_ji = -w_ij)
+//   nu_i -= m_j (l_j . d) / r^3,  nu_j += m_i (l_i . d) / r^3,  phi_i += m_j / r,  phi_j += m_i / r,
+// CTA (I, J) writes tile I's sums to partial slot J and tile J's to slot I (a diagonal CTA writes
+// both into slot I), so each body receives one write per slot; the consumer adds the NT slots in order.
+//
+// Bound by the FP64 pipe: 1/r, m_j / r^3 and m_i / r^3 come from the integer pipe as in the forward
+// loop, which with the scaled adjoints leaves 31 FP64 instructions a pair (48 when w was formed from
+// L and 1/r in FP64; N = 256: 23.9 -> 19.6 us a launch, half of it latency).
+struct AdjBody {
+  double x, y, z, m, lx, ly, lz;  // l: the velocity adjoint over the mass
+  MassSplit ms;
+  __device__ __forceinline__ void set(double x_, double y_, double z_, double m_, double Lx, double Ly, double Lz) {
+    x = x_;
+    y = y_;
+    z = z_;
+    m = m_;
+    ms = mass_split(m_);
+    const bool pad = !(m_ > 0.0);
+    lx = pad ? 0.0 : Lx / m_;
+    ly = pad ? 0.0 : Ly / m_;
+    lz = pad ? 0.0 : Lz / m_;
+  }
+};
+struct AdjSums {
+  double mux = 0.0, muy = 0.0, muz = 0.0, nu = 0.0, phi = 0.0;  // mu without the body's own mass
+};
+// Adds the pair's terms to both bodies' sums (nothing if masked).
+__device__ __forceinline__ void adj_pair(const AdjBody& a, const AdjBody& b, bool masked, AdjSums& A, AdjSums& Bs) {
+  double dx = b.x - a.x, dy = b.y - a.y, dz = b.z - a.z;
+  asm volatile("" : "+d"(dx), "+d"(dy), "+d"(dz));  // kept in registers, as in the forward loop
+  double ri, sj, si;
+  pair_scalars_int(dx, dy, dz, b.ms, a.ms, ri, sj, si);
+  ri = __longlong_as_double(masked ? 0ll : __double_as_longlong(ri));
+  sj = __longlong_as_double(masked ? 0ll : __double_as_longlong(sj));
+  si = __longlong_as_double(masked ? 0ll : __double_as_longlong(si));
+  const double pb = fma(b.lz, dz, fma(b.ly, dy, b.lx * dx)), pa = fma(a.lz, dz, fma(a.ly, dy, a.lx * dx));
+  // d . (l_b - l_a) from the differences: pb - pa would cancel where the adjoints are alike
+  const double gx = b.lx - a.lx, gy = b.ly - a.ly, gz = b.lz - a.lz;
+  const double t = -3.0 * (ri * ri) * fma(gz, dz, fma(gy, dy, gx * dx));
+  const double yx = fma(t, dx, gx), yy = fma(t, dy, gy), yz = fma(t, dz, gz);
+  A.mux = fma(sj, yx, A.mux);
+  A.muy = fma(sj, yy, A.muy);
+  A.muz = fma(sj, yz, A.muz);
+  A.nu = fma(-sj, pb, A.nu);
+  A.phi = fma(b.m, ri, A.phi);
+  Bs.mux = fma(-si, yx, Bs.mux);
+  Bs.muy = fma(-si, yy, Bs.muy);
+  Bs.muz = fma(-si, yz, Bs.muz);
+  Bs.nu = fma(si, pa, Bs.nu);
+  Bs.phi = fma(a.m, ri, Bs.phi);
+}
+
 template <int W>
 __global__ void __launch_bounds__(32 * W)
 k_adj_pair_sym(int n, int npad, int NT, int slot_lo, double G, double H, const double* __restrict__ m,
@@ -226,7 +274,7 @@ k_adj_pair_sym(int n, int npad, int NT, int slot_lo, double G, double H, const d
                const double* __restrict__ SC, double* __restrict__ mu, double* __restrict__ nu,
                double* __restrict__ phi) {
   constexpr int T = 32 * W;
-  __shared__ double sx[T], sy[T], sz[T], sm[T], slx[T], sly[T], slz[T];
+  __shared__ AdjBody sb_[T];
   __shared__ double smx[T], smy[T], smz[T], snu[T], sph[T];
   const int s = slot_lo + blockIdx.y;
   int I, J;
@@ -235,25 +283,22 @@ k_adj_pair_sym(int n, int npad, int NT, int slot_lo, double G, double H, const d
   const double* L = Lb + s * ls;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int j0 = J * T;
-  sx[tid] = R[j0 + tid];
-  sy[tid] = R[npad + j0 + tid];
-  sz[tid] = R[2 * (size_t)npad + j0 + tid];
-  sm[tid] = m[j0 + tid];
-  slx[tid] = L[j0 + tid];
-  sly[tid] = L[npad + j0 + tid];
-  slz[tid] = L[2 * (size_t)npad + j0 + tid];
+  auto body_of = [&](int q) {
+    AdjBody b;
+    b.set(R[q], R[npad + q], R[2 * (size_t)npad + q], m[q], L[q], L[npad + q], L[2 * (size_t)npad + q]);
+    return b;
+  };
+  sb_[tid] = body_of(j0 + tid);
   smx[tid] = 0.0;
   smy[tid] = 0.0;
   smz[tid] = 0.0;
   snu[tid] = 0.0;
   sph[tid] = 0.0;
   const int i = I * T + tid;
-  const double xi = R[i], yi = R[npad + i], zi = R[2 * (size_t)npad + i];
-  const double mi = m[i];
-  const double lxi = L[i], lyi = L[npad + i], lzi = L[2 * (size_t)npad + i];
+  const AdjBody bi = body_of(i);
   const bool i_pad = i >= n;
   const bool diag = (I == J);
-  double mux = 0.0, muy = 0.0, muz = 0.0, nui = 0.0, phi_i = 0.0;
+  AdjSums ai;
   __syncthreads();
 #pragma unroll 1
   for (int sb = 0; sb < W; ++sb) {
@@ -266,26 +311,13 @@ k_adj_pair_sym(int n, int npad, int NT, int slot_lo, double G, double H, const d
       for (int k = kbeg; k < kend; ++k) {
         const int jl = sub * 32 + ((lane + k) & 31);
         const bool masked = i_pad | (j0 + jl >= n) | (self & (k == 16) & (lane >= 16));
-        const double dx = sx[jl] - xi, dy = sy[jl] - yi, dz = sz[jl] - zi;
-        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        double ri = rsqrt_fp64(r2);
-        // masked pairs contribute nothing (an integer select on the bit pattern)
-        ri = __longlong_as_double(masked ? 0ll : __double_as_longlong(ri));
-        const double ri2 = ri * ri, ri3 = ri2 * ri, ri5 = ri3 * ri2;
-        const double mj = sm[jl], ljx = slx[jl], ljy = sly[jl], ljz = slz[jl];
-        const double wx = fma(mi, ljx, -mj * lxi), wy = fma(mi, ljy, -mj * lyi), wz = fma(mi, ljz, -mj * lzi);
-        const double t = 3.0 * fma(dz, wz, fma(dy, wy, dx * wx)) * ri5;
-        const double ux = fma(wx, ri3, -t * dx), uy = fma(wy, ri3, -t * dy), uz = fma(wz, ri3, -t * dz);
-        mux += ux;
-        muy += uy;
-        muz += uz;
-        smx[jl] -= ux;
-        smy[jl] -= uy;
-        smz[jl] -= uz;
-        nui = fma(-fma(ljz, dz, fma(ljy, dy, ljx * dx)), ri3, nui);
-        snu[jl] = fma(fma(lzi, dz, fma(lyi, dy, lxi * dx)), ri3, snu[jl]);
-        phi_i = fma(mj, ri, phi_i);
-        sph[jl] = fma(mi, ri, sph[jl]);
+        AdjSums aj{smx[jl], smy[jl], smz[jl], snu[jl], sph[jl]};
+        adj_pair(bi, sb_[jl], masked, ai, aj);
+        smx[jl] = aj.mux;
+        smy[jl] = aj.muy;
+        smz[jl] = aj.muz;
+        snu[jl] = aj.nu;
+        sph[jl] = aj.phi;
         __syncwarp();
       }
     }
@@ -296,16 +328,17 @@ k_adj_pair_sym(int n, int npad, int NT, int slot_lo, double G, double H, const d
   auto put = [&](int slot_of, int body, double ax_, double ay_, double az_, double n_, double p_) {
     const size_t zo = (size_t)s * NT + slot_of;
     double* muo = mu + zo * st;
-    muo[body] = gg * ax_;
-    muo[npad + body] = gg * ay_;
-    muo[2 * (size_t)npad + body] = gg * az_;
+    const double gm = gg * m[body];
+    muo[body] = gm * ax_;
+    muo[npad + body] = gm * ay_;
+    muo[2 * (size_t)npad + body] = gm * az_;
     nu[zo * npad + body] = gg * n_;
     phi[zo * npad + body] = G * p_;
   };
   if (diag) {
-    put(I, i, mux + smx[tid], muy + smy[tid], muz + smz[tid], nui + snu[tid], phi_i + sph[tid]);
+    put(I, i, ai.mux + smx[tid], ai.muy + smy[tid], ai.muz + smz[tid], ai.nu + snu[tid], ai.phi + sph[tid]);
   } else {
-    put(J, i, mux, muy, muz, nui, phi_i);
+    put(J, i, ai.mux, ai.muy, ai.muz, ai.nu, ai.phi);
     put(I, j0 + tid, smx[tid], smy[tid], smz[tid], snu[tid], sph[tid]);
   }
 }
@@ -320,9 +353,10 @@ k_adj_pair_sym_ks(int n, int npad, int NT, int slot_lo, double G, double H, cons
                   const double* __restrict__ SC, double* __restrict__ mu, double* __restrict__ nu,
                   double* __restrict__ phi) {
   constexpr int T = 32;
-  __shared__ double sx[T], sy[T], sz[T], sm[T], slx[T], sly[T], slz[T];
-  __shared__ double smx[S][T], smy[S][T], smz[S][T], snu[S][T], sph[S][T];  // partner sums per warp
-  __shared__ double rmx[S][T], rmy[S][T], rmz[S][T], rnu[S][T], rph[S][T];  // i-side sums per warp
+  __shared__ AdjBody sb_[T];
+  __shared__ double sj5[S][5][T];  // partner sums per warp: mu (3), nu, phi
+  __shared__ double si5[S][5][T];  // i-side sums per warp
+  __shared__ double s_gg;
   const int s = slot_lo + blockIdx.y;
   int I, J;
   tile_pair(blockIdx.x, NT, I, J);
@@ -330,93 +364,71 @@ k_adj_pair_sym_ks(int n, int npad, int NT, int slot_lo, double G, double H, cons
   const double* L = Lb + s * ls;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int j0 = J * T;
-  if (warp == 0) {
-    sx[lane] = R[j0 + lane];
-    sy[lane] = R[npad + j0 + lane];
-    sz[lane] = R[2 * (size_t)npad + j0 + lane];
-    sm[lane] = m[j0 + lane];
-    slx[lane] = L[j0 + lane];
-    sly[lane] = L[npad + j0 + lane];
-    slz[lane] = L[2 * (size_t)npad + j0 + lane];
-  }
-  smx[warp][lane] = 0.0;
-  smy[warp][lane] = 0.0;
-  smz[warp][lane] = 0.0;
-  snu[warp][lane] = 0.0;
-  sph[warp][lane] = 0.0;
+  auto body_of = [&](int q) {
+    AdjBody b;
+    b.set(R[q], R[npad + q], R[2 * (size_t)npad + q], m[q], L[q], L[npad + q], L[2 * (size_t)npad + q]);
+    return b;
+  };
+  // each tile's bodies once (a quotient each), by two of the warps
+  __shared__ AdjBody sa_[T];
   const int i = I * T + lane;
-  const double xi = R[i], yi = R[npad + i], zi = R[2 * (size_t)npad + i];
-  const double mi = m[i];
-  const double lxi = L[i], lyi = L[npad + i], lzi = L[2 * (size_t)npad + i];
+  if (warp == 0) sb_[lane] = body_of(j0 + lane);
+  if (warp == 1) sa_[lane] = body_of(i);
+  if (tid == 32 * S - 1) s_gg = G * (H / (double)(2 * (s + 1))) / SC[s * kScal + SC_U];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) sj5[warp][c][lane] = 0.0;
   const bool i_pad = i >= n;
   const bool diag = (I == J);
   const int kbeg = diag ? 1 + 16 * warp / S : 32 * warp / S;
   const int kend = diag ? 1 + 16 * (warp + 1) / S : 32 * (warp + 1) / S;
-  double mux = 0.0, muy = 0.0, muz = 0.0, nui = 0.0, phi_i = 0.0;
+  AdjSums ai;
   __syncthreads();
+  const AdjBody bi = sa_[lane];
 #pragma unroll 2
   for (int k = kbeg; k < kend; ++k) {
     const int jl = (lane + k) & 31;
     const bool masked = i_pad | (j0 + jl >= n) | (diag & (k == 16) & (lane >= 16));
-    const double dx = sx[jl] - xi, dy = sy[jl] - yi, dz = sz[jl] - zi;
-    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    double ri = rsqrt_fp64(r2);
-    ri = __longlong_as_double(masked ? 0ll : __double_as_longlong(ri));
-    const double ri2 = ri * ri, ri3 = ri2 * ri, ri5 = ri3 * ri2;
-    const double mj = sm[jl], ljx = slx[jl], ljy = sly[jl], ljz = slz[jl];
-    const double wx = fma(mi, ljx, -mj * lxi), wy = fma(mi, ljy, -mj * lyi), wz = fma(mi, ljz, -mj * lzi);
-    const double t = 3.0 * fma(dz, wz, fma(dy, wy, dx * wx)) * ri5;
-    const double ux = fma(wx, ri3, -t * dx), uy = fma(wy, ri3, -t * dy), uz = fma(wz, ri3, -t * dz);
-    mux += ux;
-    muy += uy;
-    muz += uz;
-    smx[warp][jl] -= ux;
-    smy[warp][jl] -= uy;
-    smz[warp][jl] -= uz;
-    nui = fma(-fma(ljz, dz, fma(ljy, dy, ljx * dx)), ri3, nui);
-    snu[warp][jl] = fma(fma(lzi, dz, fma(lyi, dy, lxi * dx)), ri3, snu[warp][jl]);
-    phi_i = fma(mj, ri, phi_i);
-    sph[warp][jl] = fma(mi, ri, sph[warp][jl]);
+    double* q = &sj5[warp][0][jl];
+    AdjSums aj{q[0], q[T], q[2 * T], q[3 * T], q[4 * T]};
+    adj_pair(bi, sb_[jl], masked, ai, aj);
+    q[0] = aj.mux;
+    q[T] = aj.muy;
+    q[2 * T] = aj.muz;
+    q[3 * T] = aj.nu;
+    q[4 * T] = aj.phi;
     __syncwarp();
   }
-  rmx[warp][lane] = mux;
-  rmy[warp][lane] = muy;
-  rmz[warp][lane] = muz;
-  rnu[warp][lane] = nui;
-  rph[warp][lane] = phi_i;
+  double* q = &si5[warp][0][lane];
+  q[0] = ai.mux;
+  q[T] = ai.muy;
+  q[2 * T] = ai.muz;
+  q[3 * T] = ai.nu;
+  q[4 * T] = ai.phi;
   __syncthreads();
-  if (warp != 0) return;
-  double ax = rmx[0][lane], ay = rmy[0][lane], az = rmz[0][lane], an = rnu[0][lane], ap = rph[0][lane];
-  double bx = smx[0][lane], by = smy[0][lane], bz = smz[0][lane], bn = snu[0][lane], bp = sph[0][lane];
-#pragma unroll
-  for (int w = 1; w < S; ++w) {
-    ax += rmx[w][lane];
-    ay += rmy[w][lane];
-    az += rmz[w][lane];
-    an += rnu[w][lane];
-    ap += rph[w][lane];
-    bx += smx[w][lane];
-    by += smy[w][lane];
-    bz += smz[w][lane];
-    bn += snu[w][lane];
-    bp += sph[w][lane];
-  }
-  const double gg = G * (H / (double)(2 * (s + 1))) / SC[s * kScal + SC_U];
+  // warp c (round robin) adds sum c of the S copies and writes it
   const size_t st = (size_t)3 * npad;
-  auto put = [&](int slot_of, int body, double ax_, double ay_, double az_, double n_, double p_) {
-    const size_t zo = (size_t)s * NT + slot_of;
-    double* muo = mu + zo * st;
-    muo[body] = gg * ax_;
-    muo[npad + body] = gg * ay_;
-    muo[2 * (size_t)npad + body] = gg * az_;
-    nu[zo * npad + body] = gg * n_;
-    phi[zo * npad + body] = G * p_;
-  };
-  if (diag) {
-    put(I, i, ax + bx, ay + by, az + bz, an + bn, ap + bp);
-  } else {
-    put(J, i, ax, ay, az, an, ap);
-    put(I, j0 + lane, bx, by, bz, bn, bp);
+  for (int c = warp; c < 5; c += S) {
+    double va = si5[0][c][lane], vb = sj5[0][c][lane];
+#pragma unroll
+    for (int w = 1; w < S; ++w) {
+      va += si5[w][c][lane];
+      vb += sj5[w][c][lane];
+    }
+    auto put = [&](int slot_of, int body, double m_, double x) {
+      const size_t zo = (size_t)s * NT + slot_of;
+      if (c < 3)
+        mu[zo * st + (size_t)c * npad + body] = s_gg * m_ * x;
+      else if (c == 3)
+        nu[zo * npad + body] = s_gg * x;
+      else
+        phi[zo * npad + body] = G * x;
+    };
+    if (diag) {
+      put(I, i, bi.m, va + vb);
+    } else {
+      put(J, i, bi.m, va);
+      put(I, j0 + lane, sb_[lane].m, vb);
+    }
   }
 }
 
@@ -429,20 +441,23 @@ k_adj_kick(int n, int npad, int slot_lo, double H, const double* __restrict__ m,
            double* __restrict__ lm) {
   __shared__ double s_lg;
   const int s = slot_lo + blockIdx.y;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t st = (size_t)3 * npad;
+  double mc[3] = {0.0, 0.0, 0.0}, nv = 0.0, ph = 0.0;
+  if (i < n) {
+#pragma unroll 4
+    for (int z = 0; z < nz; ++z) {  // four slots' loads in flight: their latency bounds the launch
+      const size_t zo = (size_t)s * nz + z;
+      for (int c = 0; c < 3; ++c) mc[c] += mu[zo * st + (size_t)c * npad + i];
+      nv += nu[zo * npad + i];
+      ph += phi[zo * npad + i];
+    }
+  }
   sum_partials(pg + (size_t)s * nblk, nblk, 1, &s_lg);
   const double U = SC[s * kScal + SC_U];
   const double delta = H / (double)(2 * (s + 1));
   const double lU = -s_lg * delta / (U * U);
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const size_t st = (size_t)3 * npad;
-  double mc[3] = {0.0, 0.0, 0.0}, nv = 0.0, ph = 0.0;
-  for (int z = 0; z < nz; ++z) {
-    const size_t zo = (size_t)s * nz + z;
-    for (int c = 0; c < 3; ++c) mc[c] += mu[zo * st + (size_t)c * npad + i];
-    nv += nu[zo * npad + i];
-    ph += phi[zo * npad + i];
-  }
   for (int c = 0; c < 3; ++c) {
     const size_t o = s * st + (size_t)c * npad + i;
     lr[o] += mc[c] + lU * m[i] * A[o];
