@@ -595,9 +595,10 @@ k_substep_cluster(int n, int npad, int nblk, int slot_lo, int pos_lo, int tau, c
   }
 }
 
-// Sum over a warp (lane 0 holds it): a fixed shuffle tree.
-__device__ __forceinline__ double warp_sum(double x) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+// Sum over the first 2 half lanes of a warp (lane 0 holds it; the others add zeros): a fixed shuffle
+// tree.
+__device__ __forceinline__ double warp_sum(double x, int half) {
+  for (int o = half; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
   return x;
 }
 
@@ -698,6 +699,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
   double t_phys = t0 + f0, T = T0, U = 0.0;
   __syncthreads();
 
+  const int half = n >= 32 ? 16 : (n > 1 ? 1 << (31 - __clz(n - 1)) : 0);  // steps of the sums over a warp's bodies
   // Cartesian vectors of the edge vectors W (one component per task) by path sums
   auto path_sum = [&](const double* W) {
     double q = 0.0;
@@ -715,7 +717,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
   auto velocities = [&]() {
     double q = path_sum(V);
     if (task) {  // warp-uniform (3 npad is a multiple of 32)
-      const double s = warp_sum(__dmul_rn(mv, q));
+      const double s = warp_sum(__dmul_rn(mv, q), half);
       if (lane == 0) red[warp] = s;
     }
     __syncthreads();
@@ -737,7 +739,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
   // of substep tau, to every thread (s_val[3], s_val[0])
   auto kinetic = [&](double x, int tau) {
     if (task) {
-      const double s = warp_sum(x);
+      const double s = warp_sum(x, half);
       if (lane == 0) red[warp] = s;
     }
     __syncthreads();
@@ -761,17 +763,71 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
   S = S < 1 ? 1 : (S > 8 ? 8 : S);
   const int ntask = ntp * S;  // <= kDivisionCtaTasks C (ntp <= 15)
   const bool nd1 = n_d >= 1, nd2 = n_d >= 2;
+  // What the tree alone decides is found once: the task's tiles and steps, the pairs to leave out (bit
+  // k - kb of mw), the steps with a pair in any lane (live: none in systems of three bodies), and the
+  // near partners of body i that fall to the task: number share, share + count, ... of its list
+  // (parent, children, grandparent, grandchildren, siblings), the first of them packed in near0.
+  const int w = rank + C * warp;  // the warp's task
+  int I = 0, J = 0, kb = 0, ke = 0;
+  if (w < ntask) {
+    const int tp = w / S, sc_ = w - (w / S) * S;
+    tile_pair(tp, nb, I, J);
+    kb = I == J ? 1 + (16 * sc_) / S : (32 * sc_) / S;
+    ke = I == J ? 1 + (16 * (sc_ + 1)) / S : (32 * (sc_ + 1)) / S;
+  }
+  const bool diag = I == J;
+  const int i = 32 * I + lane, j0 = 32 * J;
+  const bool i_pad = i >= n;
+  unsigned mw = 0u, live = 0u;
+  int nnear = 0, near0 = 0;  // partners in the list, 0 for a body of no task
+  const int count = (nb - I) * S, share = w < ntask ? (J - I) * S + w % S : 0;
+  // partner t of body i's list: its index, the edge vectors a and b (b + 1; 0: none) whose sum is the
+  // separation, and their signs
+  auto partner = [&](int t) {
+    auto pack = [](int q, int a, bool na, int b, bool nb_) {
+      return q | a << 8 | (b + 1) << 16 | (na ? 1 << 24 : 0) | (nb_ ? 1 << 25 : 0);
+    };
+    const int pi = sP[i], c0 = sCo[i], nc = sCo[i + 1] - c0;
+    if (pi >= 0 && t-- == 0) return pack(pi, i, true, -1, false);
+    if (t < nc) return pack(sCi[c0 + t], sCi[c0 + t], false, -1, false);
+    t -= nc;
+    if (sG[i] >= 0 && t-- == 0) return pack(sG[i], i, true, pi, true);
+    for (int q = c0; q < c0 + nc; ++q) {
+      const int ch = sCi[q], g0 = sCo[ch], g = sCo[ch + 1] - g0;
+      if (t < g) return pack(sCi[g0 + t], sCi[g0 + t], false, ch, false);
+      t -= g;
+    }
+    int q = sCo[pi];
+    for (; sCi[q] == i || t-- > 0; ++q) {
+    }
+    return pack(sCi[q], sCi[q], false, i, true);
+  };
+  if (w < ntask) {
+    const int pi = sP[i], gpi = sG[i];
+    for (int k = kb; k < ke; ++k) {
+      const int j = j0 + ((lane + k) & 31), pj = sP[j], gj = sG[j];
+      bool masked = i_pad | (j >= n) | (diag & (k == 16) & (lane >= 16));
+      masked |= nd1 & ((pi == j) | (pj == i));
+      masked |= nd2 & ((gpi == j) | (gj == i) | (pi == pj));
+      mw |= masked ? 1u << (k - kb) : 0u;
+      live |= masked ? 0u : 1u << (k - kb);
+    }
+    live = __reduce_or_sync(0xffffffffu, live);
+    if (nd1 && !i_pad) {
+      const int c0 = sCo[i], c1 = sCo[i + 1];
+      nnear = (pi >= 0) + c1 - c0;
+      if (nd2) {
+        nnear += gpi >= 0;
+        for (int q = c0; q < c1; ++q) nnear += sCo[sCi[q] + 1] - sCo[sCi[q]];
+        if (pi >= 0) nnear += sCo[pi + 1] - sCo[pi] - 1;
+      }
+      if (share < nnear) near0 = partner(share);
+    }
+  }
   for (int tau = 1; tau <= nk; ++tau) {
     double* partb = part + (size_t)(tau & 1) * kDivisionCtaTasks * 7 * 32;  // this substep's buffer
     __syncthreads();  // sx holds the rebuilt positions
-    const int w = rank + C * warp;  // the warp's task
     if (w < ntask) {
-      const int tp = w / S, sc_ = w - (w / S) * S;
-      int I, J;
-      tile_pair(tp, nb, I, J);
-      const bool diag = I == J;
-      const int kb = diag ? 1 + (16 * sc_) / S : (32 * sc_) / S;
-      const int ke = diag ? 1 + (16 * (sc_ + 1)) / S : (32 * (sc_ + 1)) / S;
       double* pt = partb + (size_t)warp * 7 * 32;  // the task's 7 planes
       double* jx = pt + 4 * 32;
       double* jy = jx + 32;
@@ -780,11 +836,8 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
       jy[lane] = 0.0;
       jz[lane] = 0.0;
       __syncwarp();
-      const int i = 32 * I + lane, j0 = 32 * J;
       const double xi = sx[i], yi = sx[npad + i], zi = sx[2 * npad + i];
       const MassSplit msi{smm[i], sme[i]};
-      const int pi = sP[i], gpi = sG[i];
-      const bool i_pad = i >= n;
       double ax = 0.0, ay = 0.0, az = 0.0;
       UAcc uacc;
       bool ubad = false;
@@ -792,11 +845,9 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
       int eR;
       double sj, si;
       for (int k = kb; k < ke; ++k) {
+        if (!((live >> (k - kb)) & 1u)) continue;
         const int jl = (lane + k) & 31, j = j0 + jl;
-        const int pj = sP[j], gj = sG[j];
-        bool masked = i_pad | (j >= n) | (diag & (k == 16) & (lane >= 16));
-        masked |= nd1 & ((pi == j) | (pj == i));
-        masked |= nd2 & ((gpi == j) | (gj == i) | (pi == pj));
+        const bool masked = (mw >> (k - kb)) & 1u;
         const double dx = sx[j] - xi, dy = sx[npad + j] - yi, dz = sx[2 * npad + j] - zi;
         const unsigned long long mjm = smm[j];
         const int mje = sme[j];
@@ -815,54 +866,29 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
         __syncwarp();
       }
       // this task's share of body i's near partners: separation d = r_q - r_i from the edge
-      // vectors, (+-X_a) + (+-X_b) (no second term for b < 0), signs flipped on the bit patterns
-      if (nd1 && !i_pad) {
-        const int count = (nb - I) * S, share = (J - I) * S + sc_;
-        int kc = 0;  // partners seen so far, mod count
-        const double* Xx = X;
-        const double* Xy = X + npad;
-        const double* Xz = X + 2 * (size_t)npad;
+      // vectors, (+-X_a) + (+-X_b) (no second term without b), signs flipped on the bit patterns. The
+      // lanes evaluate whatever partner each has together: by kind of partner, in turn, the slowest
+      // warp took some 12000 cycles of a substep's 33000 at N = 32 and 64
+      for (int t = share; __any_sync(0xffffffffu, t < nnear); t += count) {
+        if (t >= nnear) continue;
+        const int e = t == share ? near0 : partner(t);
+        const int q = e & 255, ea = (e >> 8) & 255, eb = ((e >> 16) & 255) - 1;
         auto flip = [](double x, bool neg) {
           return neg ? __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull) : x;
         };
-        auto near = [&](int q, int a, bool na, int b, bool nb_) {
-          const bool mine = kc == share;
-          kc = kc + 1 == count ? 0 : kc + 1;
-          if (!mine) return;
-          double dx = flip(Xx[a], na), dy = flip(Xy[a], na), dz = flip(Xz[a], na);
-          if (b >= 0) {
-            dx = __dadd_rn(dx, flip(Xx[b], nb_));
-            dy = __dadd_rn(dy, flip(Xy[b], nb_));
-            dz = __dadd_rn(dz, flip(Xz[b], nb_));
-          }
-          pair_scalars_core(dx, dy, dz, MassSplit{smm[q], sme[q]}, msi, Rn, eR, sj, si);
-          ubad |= Rn == 0ull;
-          ax = fma(sj, dx, ax);
-          ay = fma(sj, dy, ay);
-          az = fma(sj, dz, az);
-          if (q > i) uacc.add(__umul64hi(smm[q], Rn), sme[q] + eR + 64);
-        };
-        if (pi >= 0) near(pi, i, true, -1, false);
-        const int c0 = sCo[i], c1 = sCo[i + 1];
-        for (int a = c0; a < c1; ++a) {
-          const int ch = sCi[a];
-          near(ch, ch, false, -1, false);
+        const bool na = (e >> 24) & 1, nb_ = (e >> 25) & 1;
+        double dx = flip(X[ea], na), dy = flip(X[npad + ea], na), dz = flip(X[2 * npad + ea], na);
+        if (eb >= 0) {
+          dx = __dadd_rn(dx, flip(X[eb], nb_));
+          dy = __dadd_rn(dy, flip(X[npad + eb], nb_));
+          dz = __dadd_rn(dz, flip(X[2 * npad + eb], nb_));
         }
-        if (nd2) {
-          if (gpi >= 0) near(gpi, i, true, pi, true);
-          for (int a = c0; a < c1; ++a) {
-            const int ch = sCi[a];
-            for (int b = sCo[ch]; b < sCo[ch + 1]; ++b) {
-              const int gc = sCi[b];
-              near(gc, gc, false, ch, false);
-            }
-          }
-          if (pi >= 0)
-            for (int b = sCo[pi]; b < sCo[pi + 1]; ++b) {
-              const int sb = sCi[b];
-              if (sb != i) near(sb, sb, false, i, true);
-            }
-        }
+        pair_scalars_core(dx, dy, dz, MassSplit{smm[q], sme[q]}, msi, Rn, eR, sj, si);
+        ubad |= Rn == 0ull;
+        ax = fma(sj, dx, ax);
+        ay = fma(sj, dy, ay);
+        az = fma(sj, dz, az);
+        if (q > i) uacc.add(__umul64hi(smm[q], Rn), sme[q] + eR + 64);
       }
       const double ui = ubad ? __longlong_as_double(0x7ff8000000000000LL) : uacc.value();
       if (diag) {  // both sides belong to tile I's bodies
@@ -932,7 +958,7 @@ k_division_cta(int n, int npad, int K, int n_d, double G, const double* __restri
     }
     {
       if (warp < nb) {
-        const double s = warp_sum(um);
+        const double s = warp_sum(um, half);
         if (lane == 0) red[warp] = s;
       }
       __syncthreads();
