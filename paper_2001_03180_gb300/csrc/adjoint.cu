@@ -433,7 +433,7 @@ k_adj_pair_sym_ks(int n, int npad, int NT, int slot_lo, double G, double H, cons
 }
 
 // Transposed kick of level tau: lU from the lv . a partials, then lr += mu + lU m a and
-// lm += nu + lU phi (mu, nu, phi summed over their nz partial slots in order).
+// lm += nu + lU phi (mu, nu, phi summed over their nz partial slots in order, four at a time by pairs).
 __global__ void __launch_bounds__(kBlock)
 k_adj_kick(int n, int npad, int slot_lo, double H, const double* __restrict__ m, const double* __restrict__ A,
            const double* __restrict__ SC, const double* __restrict__ pg, int nblk, const double* __restrict__ mu,
@@ -445,8 +445,21 @@ k_adj_kick(int n, int npad, int slot_lo, double H, const double* __restrict__ m,
   const size_t st = (size_t)3 * npad;
   double mc[3] = {0.0, 0.0, 0.0}, nv = 0.0, ph = 0.0;
   if (i < n) {
-#pragma unroll 4
-    for (int z = 0; z < nz; ++z) {  // four slots' loads in flight: their latency bounds the launch
+    int z = 0;
+    for (; z + 4 <= nz; z += 4) {  // four slots' loads in flight: their latency bounds the launch
+      double b[4][5];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const size_t zo = (size_t)s * nz + z + k;
+        for (int c = 0; c < 3; ++c) b[k][c] = mu[zo * st + (size_t)c * npad + i];
+        b[k][3] = nu[zo * npad + i];
+        b[k][4] = phi[zo * npad + i];
+      }
+      for (int c = 0; c < 3; ++c) mc[c] += (b[0][c] + b[1][c]) + (b[2][c] + b[3][c]);
+      nv += (b[0][3] + b[1][3]) + (b[2][3] + b[3][3]);
+      ph += (b[0][4] + b[1][4]) + (b[2][4] + b[3][4]);
+    }
+    for (; z < nz; ++z) {
       const size_t zo = (size_t)s * nz + z;
       for (int c = 0; c < 3; ++c) mc[c] += mu[zo * st + (size_t)c * npad + i];
       nv += nu[zo * npad + i];

@@ -3,9 +3,8 @@
 // Far pairs use Cartesian separations r_j - r_i; near pairs (within N_d tree edges,
 // Eq. LCA) use sums of MST edge vectors. The tiled kernel evaluates every unordered far
 // pair exactly once and applies the result to both bodies (a_i += m_j d/r^3,
-// a_j -= m_i d/r^3), which halves the FP64 work - the resource that bounds this loop on
-// GB300. Near pairs are masked out of the tiles with integer compares on parent and
-// grandparent indices and summed in a sparse pass with the edge-vector separations.
+// a_j -= m_i d/r^3), which halves the work. Near pairs are masked out of the tiles (by words that
+// the tree gives) and summed in a sparse pass with the edge-vector separations.
 //
 // Two arithmetics, chosen per pair of 32-body sub-tiles:
 //  - integer (pairint.cuh): the whole interaction on the integer and FP32 pipes, accumulated in
@@ -57,7 +56,8 @@
 namespace mstar {
 namespace {
 
-// Sum of tile t's NT partial slots (ascending s) for its T bodies, one per thread of the
+// Sum of tile t's NT partial slots (ascending s, four at a time by pairs: a chain a quarter as long,
+// in time and in roundings) for its T bodies, one per thread of the
 // first T of the CTA's NTH threads, into Pt (4 planes); then its count is reset and the
 // partials' lines dropped from L2. Every thread of the CTA calls it (it holds a barrier).
 template <int T, int NTH = T>
@@ -67,7 +67,7 @@ __device__ __forceinline__ void finish_tile(int t, int npad, int NT, const doubl
     const double* q = Ps + (size_t)t * T + tid;
     double ax = 0.0, ay = 0.0, az = 0.0, u = 0.0;
     // L2 loads (the slots were written by other CTAs after this SM's L1 could have seen
-    // them), four slots at a time ahead of their additions, which keep the ascending order
+    // them), four slots at a time ahead of their additions
     int s = 0;
     for (; s + 4 <= NT; s += 4) {
       double b[4][4];
@@ -79,13 +79,10 @@ __device__ __forceinline__ void finish_tile(int t, int npad, int NT, const doubl
         b[k][2] = __ldcg(qs + 2 * (size_t)npad);
         b[k][3] = __ldcg(qs + 3 * (size_t)npad);
       }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        ax += b[k][0];
-        ay += b[k][1];
-        az += b[k][2];
-        u += b[k][3];
-      }
+      ax += (b[0][0] + b[1][0]) + (b[2][0] + b[3][0]);
+      ay += (b[0][1] + b[1][1]) + (b[2][1] + b[3][1]);
+      az += (b[0][2] + b[1][2]) + (b[2][2] + b[3][2]);
+      u += (b[0][3] + b[1][3]) + (b[2][3] + b[3][3]);
     }
     for (; s < NT; ++s) {
       const double* qs = q + (size_t)s * 4 * npad;
@@ -505,8 +502,7 @@ k_pair_finish(int n, int npad, int NT, int slot_lo, int n_d, double G, const dou
         double t[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) t[k] = q[(size_t)(s + k) * 4 * npad];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc += t[k];
+        acc += (t[0] + t[1]) + (t[2] + t[3]);
       }
       for (; s < NT; ++s) acc += q[(size_t)s * 4 * npad];
     }
