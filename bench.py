@@ -38,10 +38,6 @@ FLOPS_PER_UNORDERED_PAIR = 33
 # r^2 and a Newton-refined reciprocal square root, the mass scaling, 3 DFMA accumulations, U);
 # reported beside the symmetric count.
 FLOPS_PER_ORDERED_PAIR_NONSYM = 28
-# FP64-pipe instructions the tiled kernel issues per unordered pair: 3 DADD for the separation
-# and 6 DFMA for the two force accumulations (ncu counts 3.0 DADD and 5.95 DFMA per pair).
-# r^2, 1/r, 1/r^3, the mass products and the force-function sum run on the integer pipe.
-FP64_INSTR_PER_PAIR = 9
 NOMINAL_FP64_TFLOPS = 1.25
 # FP64 FMA units: 2 DFMA per clock per SM (ncu: sm__sass_thread_inst_executed_op_dfma_pred_on
 # peak_sustained = 2 inst/cycle/SM), 152 SMs; the roofline peak is that rate at the SM clock
@@ -49,16 +45,17 @@ NOMINAL_FP64_TFLOPS = 1.25
 DFMA_PER_CLK_PER_SM = 2
 NUM_SMS = 152
 L2_FLUSH_BYTES = 256 << 20
-# Figures from ncu captures of k_pair_tiles<4> (128-body tiles) at N = 10002, each valid for the
-# kernel built from the sources whose SHA-256 (csrc/pair.cu then csrc/device.cuh) starts with
-# the given prefix; for other sources or another tile the bench reports them as null.
+# Figures from ncu captures of k_pair_tiles<4> (128-body tiles) at N = 10002, valid for the kernel
+# built from the sources whose SHA-256 (PAIR_SOURCES in order) starts with the given prefix; for
+# other sources or another tile the bench reports them as null.
 #  - DRAM bytes (read + write) of one launch by the number of division slots it evaluates;
 #    an attempt launches the kernel for 1 (step start), 8, 8, 7, 7, ..., 1, 1 slots;
-#  - the FP64 pipe's active fraction (sm__inst_executed_pipe_fp64 over its peak).
-PAIR_TILE_SRC_SHA = "54214f1fde9b5cd9"
-PAIR_TILE_PIPE_SRC_SHA = "54214f1fde9b5cd9"
-PAIR_TILE_DRAM_BYTES_BY_SLOTS = {1: 0.166e6, 2: 0.510e6, 3: 1.295e6, 4: 2.572e6, 5: 3.626e6, 6: 4.615e6, 7: 6.120e6, 8: 11.925e6}
-PAIR_TILE_FP64_PIPE_NCU = 0.870
+#  - active fractions of the pipe that takes the 32 x 32-bit products (FMA heavy) and of the FP64 pipe.
+PAIR_SOURCES = ("pair.cu", "pairtile.cuh", "pairint.cuh", "device.cuh")
+PAIR_TILE_SRC_SHA = "5467a1591a52becb"
+PAIR_TILE_DRAM_BYTES_BY_SLOTS = {}  # not captured for these sources
+PAIR_TILE_FMAHEAVY_PIPE_NCU = 0.561
+PAIR_TILE_FP64_PIPE_NCU = 0.302
 ATTEMPT_SLOT_PATTERN = [1] + [k for k in range(8, 0, -1) for _ in range(2)]
 # Algorithmic DRAM bytes of one force evaluation per body: positions 24 and mass 8 read,
 # accelerations 24 written (parent and grandparent indices are another 8 read).
@@ -70,7 +67,7 @@ def tuned_pair_loop(M, m, r, v, repeats):
     library's default) by more than 2 %, the spread of single attempts; else the size rule's."""
     best, ms = M.mstar_tune_pair_tile(m, r, v, repeats=repeats)
     n = len(m)
-    rule = (32, 4) if n <= 512 else ((32, 1) if n <= 4096 else ((64, 1) if n <= 8192 else (128, 1)))
+    rule = (32, 4) if n <= 768 else ((32, 1) if n <= 8192 else (128, 1))
     pick = best if ms[best] < 0.98 * ms[rule] else rule
     return pick, {f"{k[0]}x{k[1]}": x for k, x in ms.items()}
 
@@ -79,7 +76,7 @@ def pair_source_sha():
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("pair.cu", "device.cuh"):
+    for f in PAIR_SOURCES:
         with open(os.path.join(ROOT, "paper_2001_03180_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -672,17 +669,16 @@ def run_mstar(args):
     achieved = FLOPS_PER_UNORDERED_PAIR * pairs_per_launch / (avg_ms * 1e-3) / 1e12
     clk_mhz = clocks_prof.get("sm_mhz") or 2070.0
     fp64_peak = 2.0 * DFMA_PER_CLK_PER_SM * NUM_SMS * clk_mhz * 1e6 / 1e12
-    fp64_issue = DFMA_PER_CLK_PER_SM * NUM_SMS * clk_mhz * 1e6  # FP64 instructions/s the pipe takes
     sha_ok = pair_source_sha() == PAIR_TILE_SRC_SHA and (tile, split) == (128, 1)
     slots_per_launch = prof.force_evals / max(prof.pair_launches, 1)
     # per launch, averaged over an attempt's launches (the pattern of slot counts is fixed)
     traffic = (sum(PAIR_TILE_DRAM_BYTES_BY_SLOTS[k] for k in ATTEMPT_SLOT_PATTERN) / len(ATTEMPT_SLOT_PATTERN)
-               if sha_ok else None)
+               if sha_ok and PAIR_TILE_DRAM_BYTES_BY_SLOTS else None)
     algo_bytes = ALGO_BYTES_PER_BODY_EVAL * n * slots_per_launch
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp64_peak, "traffic": traffic,
-                "kernel": "k_pair_tiles (symmetric pair loop: FP64 separations and force accumulations; "
-                          "integer-pipe r^2, 1/r, m/r^3 and the exact fixed-point sum of m/r)",
+                "kernel": "k_pair_tiles (symmetric pair loop in 64-bit fixed point on the integer pipe; flat, "
+                          "very wide or very close tile pairs in FP64)",
                 "achieved_source": ("33 algorithmic FP64 flops per unordered far pair (each evaluated once and "
                                     "applied to both bodies) x N(N-1)/2 pairs x evaluations per launch / mean "
                                     "CUDA-event launch time on the context stream, over a second run of the "
@@ -690,14 +686,11 @@ def run_mstar(args):
                 "peak_source": ("FP64 unit peak from unit counts and clocks (no FP64 entry among the measured "
                                 "peaks): 2 DFMA/clk/SM x 152 SMs x the SM clock sampled in the timed region x "
                                 "2 flops"),
-                "frac_above_1_because": ("r^2, 1/r, r^-3, m r^-3 and the sum of m/r run on the integer pipe: the "
-                                         "FP64 pipe issues 9 instructions (3 DADD + 6 DFMA) of the 33 flops"),
-                "fp64_pipe_util": pairs_per_launch * FP64_INSTR_PER_PAIR / (avg_ms * 1e-3) / fp64_issue,
-                "fp64_pipe_util_source": ("pair rate x 9 FP64 instructions per pair / (2 per clk per SM x 152 "
-                                          "SMs x sampled clock)"),
-                "fp64_pipe_util_ncu": (PAIR_TILE_FP64_PIPE_NCU
-                                       if pair_source_sha() == PAIR_TILE_PIPE_SRC_SHA and (tile, split) == (128, 1)
-                                       else None),
+                "frac_above_1_because": ("the pairs run in 64-bit fixed point on the integer pipe: separations, r^2, "
+                                         "1/r, r^-3, mass scalings and accumulations without FP64 instructions; the "
+                                         "FP64 peak is the algorithm's yardstick, not what binds the kernel"),
+                "fma_heavy_pipe_util_ncu": PAIR_TILE_FMAHEAVY_PIPE_NCU if sha_ok else None,
+                "fp64_pipe_util_ncu": PAIR_TILE_FP64_PIPE_NCU if sha_ok else None,
                 "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum per launch by slot count, "
                                    "averaged over an attempt's 17 launches; null when the kernel's sources "
                                    "differ from the captured ones" + ("" if sha_ok else " (they differ)")),
@@ -767,7 +760,7 @@ def run_mstar(args):
         # the figures of every section in a few keys at the end of the line
         out["summary"] = {
             "abs_dE_over_E": dE_c5, "abs_dE_over_E_steps": steps_c5,
-            "roofline_frac": roofline["frac"], "fp64_pipe_util": roofline["fp64_pipe_util"],
+            "roofline_frac": roofline["frac"], "fma_heavy_pipe_util": roofline["fma_heavy_pipe_util_ncu"],
             "c1_plummer64_abs_dE_over_E": sc.get("plummer64_to_t1", {}).get("abs_dE_over_E"),
             "c1_plummer64_gbs_steps_per_s": sc.get("plummer64_to_t1", {}).get("gbs_steps_per_s"),
             "c2_smbh2050_abs_dE_over_E": sc.get("plummer2048_smbh_binary_200_steps", {}).get("abs_dE_over_E"),
