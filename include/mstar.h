@@ -87,7 +87,7 @@ typedef struct {
                         differ from the unsplit loop by rounding only. 0 */
   int division_schedule; /* how an attempt's k_fix divisions are issued: 1 level by level (the
                         kernels of a substep level for every division active at it: one CTA per
-                        division for up to 256 padded bodies, a thread-block cluster per division
+                        division for up to 160 padded bodies, a thread-block cluster per division
                         for up to 576, else one launch per kernel; all bit-identical), 2 each
                         division on its own stream (longer divisions at higher priority), so that
                         one division's small kernels overlap another's pair loop, 3 each division
