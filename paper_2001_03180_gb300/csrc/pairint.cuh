@@ -24,6 +24,10 @@
 // body's accumulators is 2^-58 of a power of two at least 1.3 times the largest force of these 32
 // partners on that body, so a sum of up to 32 terms stays below 2^63 and a term is off by at most
 // a unit: a binary64 accumulation loses 2^-54 of the running sum per term.
+// The potential m_j / r is truncated to a unit of its own, 2^-58 of a power of two at least 1.3 and at
+// most 4 times the largest m_j / r among the body's partners that are not masked, whatever the body's
+// own mass and those of the other bodies: half a unit is given back for every term, so 32 terms err
+// by at most 2^-52 of the sum together, 2^-55 typically, for any ratio of the masses.
 #pragma once
 
 #include "device.cuh"

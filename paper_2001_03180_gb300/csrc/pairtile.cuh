@@ -31,14 +31,12 @@ __device__ __forceinline__ float key_float(int k) { return __int_as_float(k ^ ((
 struct FixWindow {
   bool ok;        // the tile pair can be taken in integers
   int u;          // unit 2^u of the positions
-  int em;         // every mass < 2^em
   float inv_max;  // 1 / r^2 limit: pairs closer than 2^-10 of the extent are not taken
 };
 
-// From the extents lo[3], hi[3] of the two tiles' bodies and their largest mass exponent. The
-// float copies of the positions err by 2^-24 of the largest coordinate, which must not exceed
-// 2^8 extents, so a float r^2 of a pair at the limit is within 12 % (the limit allows for 30 %).
-__device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi, int em, bool ok) {
+// From the extents lo[3], hi[3] of the two tiles' bodies. The float copies of the positions err by
+// 2^-24 of the largest coordinate, which must not exceed 2^8 extents, so a float r^2 of a pair at the limit is within 12 % (the limit allows for 30 %).
+__device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi, bool ok) {
   FixWindow w;
   const float ext = fmaxf(hi[0] - lo[0], fmaxf(hi[1] - lo[1], hi[2] - lo[2])) * (1.0f + 0x1p-18f);
   float big = 0.0f;
@@ -47,7 +45,6 @@ __device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi
   w.ok = ok && ext >= 0x1p-30f && big <= 256.0f * ext;
   const int E = (int)((__float_as_uint(ext) >> 23) & 255u) - 126;  // ext < 2^E
   w.u = E - 62;
-  w.em = em;
   const float r = ext * 0x1p-10f;
   w.inv_max = 1.0f / (1.3f * r * r);
   return w;
@@ -64,7 +61,6 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
   const float kInf = __int_as_float(0x7f800000);
   float lo[3], hi[3];
   bool ok = true;
-  int em = -4096;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     lo[c] = fminf(i_pad ? kInf : __double2float_rd(pi3[c]), j_pad ? kInf : __double2float_rd(pj3[c]));
@@ -73,23 +69,20 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
   }
   // masses within 2^-40 ... 2^40, so that the float bounds of m / r^2 neither overflow nor vanish
   const int ei = mass_split(mi).e + 64, ej = mass_split(mj).e + 64;
-  if (!i_pad) em = ei;
-  if (!j_pad) em = max(em, ej);
   ok &= (i_pad || (ei > -40 && ei < 40)) && (j_pad || (ej > -40 && ej < 40));
   bool eq = __all_sync(0xffffffffu, (i_pad || mi == m0) && (j_pad || mj == m0));
   ok = __all_sync(0xffffffffu, ok);
-  int key[7];
+  int key[6];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     key[c] = __reduce_min_sync(0xffffffffu, float_key(lo[c]));
     key[3 + c] = __reduce_max_sync(0xffffffffu, float_key(hi[c]));
   }
-  key[6] = __reduce_max_sync(0xffffffffu, em);
   if constexpr (NW > 1) {
     if (lane == 0) {
 #pragma unroll
-      for (int c = 0; c < 7; ++c) sbox[warp][c] = key[c];
-      sbox[warp][7] = (ok ? 1 : 0) | (eq ? 2 : 0);
+      for (int c = 0; c < 6; ++c) sbox[warp][c] = key[c];
+      sbox[warp][6] = (ok ? 1 : 0) | (eq ? 2 : 0);
     }
     __syncthreads();
 #pragma unroll
@@ -99,9 +92,8 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
         key[c] = min(key[c], sbox[w][c]);
         key[3 + c] = max(key[3 + c], sbox[w][3 + c]);
       }
-      key[6] = max(key[6], sbox[w][6]);
-      ok &= (sbox[w][7] & 1) != 0;
-      eq &= (sbox[w][7] & 2) != 0;
+      ok &= (sbox[w][6] & 1) != 0;
+      eq &= (sbox[w][6] & 2) != 0;
     }
   }
 #pragma unroll
@@ -109,7 +101,7 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
     lo[c] = key_float(key[c]);
     hi[c] = key_float(key[3 + c]);
   }
-  FixWindow fw = fix_window(lo, hi, key[6], ok);
+  FixWindow fw = fix_window(lo, hi, ok);
   // The three components of a force share one unit. Where this warp's bodies lie flat (the mean
   // distance from the middle of the extent along one axis below an eighth of that along
   // another), the small component would keep fewer bits than binary64 sums do: not taken.
@@ -189,31 +181,44 @@ template <bool kPlain>
 __device__ __forceinline__ void subtile_pairs(TileBody& b, const SubTile& t, const FixWindow& fw, bool eq, double m0,
                                               unsigned mw, int k0, int k1, int lane) {
   // Float bounds of the largest force on body i (fi) and, handed from lane to lane with the
-  // partners, on each j (fj); the closest pair decides whether integers serve.
-  float fi = 0.0f, fj = 0.0f, inv_hi = 0.0f;
+  // partners, on each j (fj), and of the largest m_j / r of body i (pu); the closest pair decides
+  // whether integers serve. With equal masses the bounds leave the mass out.
+  float fi = 0.0f, fj = 0.0f, pu = 0.0f, inv_hi = 0.0f;
   if (fw.ok) {
+    if (eq) {
 #pragma unroll 4
-    for (int k = k0; k < k1; ++k) {
-      const float4 q = t.f[(lane + k) & 31];
-      const float dx = q.x - b.gx, dy = q.y - b.gy, dz = q.z - b.gz;
-      float inv = rcp_approx(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-      inv = (mw >> k) & 1u ? 0.0f : inv;
-      inv_hi = fmaxf(inv_hi, inv);
-      fi = fmaxf(fi, q.w * inv);
-      fj = fmaxf(fj, b.gm * inv);
-      fj = __shfl_sync(0xffffffffu, fj, (lane + 1) & 31);  // now of partner (lane + k + 1) mod 32
+      for (int k = k0; k < k1; ++k) {
+        const float4 q = t.f[(lane + k) & 31];
+        const float dx = q.x - b.gx, dy = q.y - b.gy, dz = q.z - b.gz;
+        float inv = rcp_approx(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+        inv = (mw >> k) & 1u ? 0.0f : inv;
+        fi = fmaxf(fi, inv);
+        fj = fmaxf(fj, inv);
+        fj = __shfl_sync(0xffffffffu, fj, (lane + 1) & 31);  // now of partner (lane + k + 1) mod 32
+      }
+      inv_hi = fi;
+      pu = sqrtf(fi);
+    } else {
+#pragma unroll 4
+      for (int k = k0; k < k1; ++k) {
+        const float4 q = t.f[(lane + k) & 31];
+        const float dx = q.x - b.gx, dy = q.y - b.gy, dz = q.z - b.gz;
+        float rinv = rsqrt_seed(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+        rinv = (mw >> k) & 1u ? 0.0f : rinv;
+        const float inv = rinv * rinv;
+        inv_hi = fmaxf(inv_hi, inv);
+        pu = fmaxf(pu, q.w * rinv);
+        fi = fmaxf(fi, q.w * inv);
+        fj = fmaxf(fj, b.gm * inv);
+        fj = __shfl_sync(0xffffffffu, fj, (lane + 1) & 31);
+      }
     }
     fj = __shfl_sync(0xffffffffu, fj, (lane - k1) & 31);  // held for partner lane + k1: to its own lane
   }
   if (__all_sync(0xffffffffu, fw.ok && inv_hi <= fw.inv_max)) {
-    if (eq) {
-      const float rm = rcp_approx(__double2float_rn(m0));
-      fi *= rm;
-      fj *= rm;
-    }
-    // accumulator units 2^L: forces below 2^58 units (the bounds hold within 1.5)
-    const int ei = (int)(__float_as_uint(1.5f * fi) >> 23) - 126, ej = (int)(__float_as_uint(1.5f * fj) >> 23) - 126;
-    const int Li = ei - 58, Lj = ej - 58, LU = (((eq ? 0 : fw.em) + ei + 1) >> 1) - 58;
+    // accumulator units 2^L: forces and potentials below 2^58 units (the bounds hold within 1.5)
+    const int Li = (int)(__float_as_uint(1.5f * fi) >> 23) - 184, Lj = (int)(__float_as_uint(1.5f * fj) >> 23) - 184,
+              LU = (int)(__float_as_uint(1.5f * pu) >> 23) - 184;
     const int cx = 116 + 2 * fw.u + (eq ? 64 : 0), ci = Li + cx, cu = LU + 60 + fw.u + (eq ? 64 : 0);
     t.cj[lane] = Lj + cx;
     t.bx[lane] = 0;
@@ -221,7 +226,8 @@ __device__ __forceinline__ void subtile_pairs(TileBody& b, const SubTile& t, con
     t.bz[lane] = 0;
     __syncwarp();
     FixAcc ai{0, 0, 0};
-    unsigned long long ui = (k1 - k0) / 2;  // the sum's shifts truncate: half a unit per term back
+    // the sum's shifts truncate: half a unit back for every term
+    unsigned long long ui = __popc(~mw & (0xffffffffu >> (32 - k1) & 0xffffffffu << k0)) / 2;
     double si = exp2_int(Li), sj = exp2_int(Lj), su = exp2_int(LU);
     if (eq) {
 #pragma unroll 2
