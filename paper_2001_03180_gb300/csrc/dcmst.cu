@@ -504,9 +504,16 @@ k_dc_nfn(int n, const int* __restrict__ ncell, const int* __restrict__ leafid, c
          const int* __restrict__ nbr, const int* __restrict__ lcount, unsigned long long* __restrict__ partD,
          int* __restrict__ partJ, int* __restrict__ flags) {
   __shared__ float4 sq[kDcT];
-  __shared__ int s_emax;
-  if (flags[0] != 0 || flags[1] >= n - *ncell) return;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) flags[3] += 1;
+  __shared__ int s_emax, s_stop;
+  if (threadIdx.x == 0) {
+    // read once: other CTAs of this launch may set the tie flag meanwhile, and a CTA whose warps saw
+    // different values would go on with part of its warps
+    s_stop = flags[0] != 0 || flags[1] >= n - *ncell;
+    s_emax = 0;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && !s_stop) flags[3] += 1;
+  }
+  __syncthreads();
+  if (s_stop) return;
   const int p0 = blockIdx.x * kDcT, p = p0 + threadIdx.x, q = blockIdx.y;
   const int u_lo = leaf_start[leafid[p0]], u_hi = leaf_start[leafid[min(n, p0 + kDcT) - 1] + 1];
   const int per = (u_hi - u_lo + kDcParts - 1) / kDcParts;
@@ -521,7 +528,6 @@ k_dc_nfn(int n, const int* __restrict__ ncell, const int* __restrict__ leafid, c
     const int b = nbr[p];
     need = lcount[g] < leaf_start[g + 1] - leaf_start[g] - 1 && (b < 0 || comp[b] == cp);
   }
-  if (threadIdx.x == 0) s_emax = 0;
   if (!__syncthreads_or(need)) return;
   const float4 fp = p < n ? sf4[p] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   NearestScan ns;
@@ -609,13 +615,17 @@ k_dc_round(int n, const int* __restrict__ ncell, const int* __restrict__ leaf_st
            const unsigned long long* __restrict__ sorted, int* comp, int* nbr, unsigned long long* nbrD, int* cidx,
            int* nxt, const unsigned long long* __restrict__ partD, const int* __restrict__ partJ,
            unsigned long long* cmin, int* lcount, int* __restrict__ eu, int* __restrict__ ev, int* flags) {
-  __shared__ int s_tie, s_edges;
+  __shared__ int s_tie, s_edges, s_stop;
   const int g = blockIdx.x;
-  if (g >= *ncell || flags[0] != 0) return;
+  if (g >= *ncell) return;
   const int lo = leaf_start[g], hi = leaf_start[g + 1];
+  if (threadIdx.x == 0) {
+    s_stop = flags[0];  // read once, as in the search: it may change during the launch
+    s_tie = s_edges = 0;
+  }
+  __syncthreads();
   const int done = lcount[g];
-  if (done >= hi - lo - 1) return;
-  if (threadIdx.x == 0) s_tie = s_edges = 0;
+  if (s_stop || done >= hi - lo - 1) return;
   for (int p = lo + threadIdx.x; p < hi; p += kDcRoundT) {
     cmin[p] = ~0ull;
     cidx[p] = -1;
