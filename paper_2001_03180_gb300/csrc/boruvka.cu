@@ -42,15 +42,15 @@ k_nfn(int n, int npad, int nparts, const double* __restrict__ X, const double* _
       const double* __restrict__ Z, const float* __restrict__ f4, const int* __restrict__ comp,
       const int* __restrict__ nbr, unsigned long long* __restrict__ partD, int* __restrict__ partJ,
       int* __restrict__ flags) {
-  // The round's gate: flags[2] = 1 once the tree is complete (flags[1] = n - 1 edges, written
-  // by the previous round's k_hook) or a tie has been seen (flags[0]); the round's kernels then
+  // The round's gate: flags[4] = 1 once the tree is complete (flags[1] = n - 1 edges) or a tie has
+  // been seen (flags[0]), decided by the last kernel of the previous round; the round's kernels then
   // return at once, and flags[3] counts the rounds that ran. Rounds can thus be issued ahead of
   // the host's check: a round after the last one needed changes nothing (without the gate it
-  // would find no foreign neighbour and report a tie). The search opens every round, so its
-  // first CTA publishes the decision for the round's later kernels (none of which writes
-  // flags[2]). A tie set by another CTA while the search runs can make CTAs decide differently;
-  // the build then falls back to the Prim kernel, so nothing of that round is used.
-  const bool stop = (flags[0] != 0) || (flags[1] >= n - 1);
+  // would find no foreign neighbour and report a tie). No kernel of the round writes flags[4]
+  // before k_relabel, so every CTA of the search decides alike: a tie found while it runs ends the
+  // build after this round, whose other kernels still get a neighbour for every vertex. The search's
+  // first CTA copies the gate to flags[2] for them.
+  const bool stop = flags[4] != 0;
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
     flags[2] = stop;
     if (!stop) flags[3] += 1;
@@ -234,10 +234,12 @@ __global__ void k_hook(int n, const int* __restrict__ comp, const int* __restric
   }
 }
 
+// The new labels, and the next round's gate.
 __global__ void k_relabel(int n, int* __restrict__ comp, const int* __restrict__ nxt,
-                          unsigned long long* __restrict__ cmin, int* __restrict__ ccnt, const int* __restrict__ stop) {
+                          unsigned long long* __restrict__ cmin, int* __restrict__ ccnt, int* __restrict__ flags) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || *stop) return;
+  if (i >= n || flags[2]) return;
+  if (i == 0) flags[4] = flags[0] != 0 || flags[1] >= n - 1;
   int c = comp[i];
   for (int guard = 0; guard < n && nxt[c] != c; ++guard) c = nxt[c];
   comp[i] = c;
@@ -514,7 +516,8 @@ cudaError_t launch_mst_boruvka(mstar_ctx* c, bool* tied) {
   int* ev = reinterpret_cast<int*>(take(sizeof(int) * npad));
   unsigned long long* partD = reinterpret_cast<unsigned long long*>(take(8 * (size_t)npad * nparts));
   int* partJ = reinterpret_cast<int*>(take(sizeof(int) * (size_t)npad * nparts));
-  int* flags = reinterpret_cast<int*>(take(sizeof(int) * 4));  // [0] tie, [1] edge count, [2] gate, [3] rounds run
+  int* flags = reinterpret_cast<int*>(take(sizeof(int) * 5));  // [0] tie, [1] edge count, [2] gate of the round,
+                                                               // [3] rounds run, [4] gate of the next
   const size_t p_bytes = (size_t)c->nslots * c->NT * 4 * npad * sizeof(double);
   if ((size_t)(base - reinterpret_cast<char*>(c->d.P)) > p_bytes) {  // scratch does not fit: use Prim
     *tied = true;
@@ -524,7 +527,7 @@ cudaError_t launch_mst_boruvka(mstar_ctx* c, bool* tied) {
   const double* Y = X + npad;
   const double* Z = Y + npad;
   const int nb = (n + 255) / 256;
-  cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * 4, c->stream);
+  cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * 5, c->stream);
   if (e != cudaSuccess) return e;
   k_boruvka_init<<<nb, 256, 0, c->stream>>>(n, X, Y, Z, f4, comp, nbr, cmin, ccnt);
   MSTAR_LAUNCHED(c);
@@ -543,7 +546,7 @@ cudaError_t launch_mst_boruvka(mstar_ctx* c, bool* tied) {
       k_comp_min<<<nb, 256, 0, c->stream>>>(n, comp, nbrD, cmin, flags + 2);
       k_comp_edge<<<nb, 256, 0, c->stream>>>(n, comp, nbrD, cmin, cidx, ccnt, flags, flags + 2);
       k_hook<<<nb, 256, 0, c->stream>>>(n, comp, nbr, cidx, nxt, eu, ev, flags + 1, flags + 2);
-      k_relabel<<<nb, 256, 0, c->stream>>>(n, comp, nxt, cmin, ccnt, flags + 2);
+      k_relabel<<<nb, 256, 0, c->stream>>>(n, comp, nxt, cmin, ccnt, flags);
       c->launches += 6;
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -48,3 +48,20 @@ def test_divide_and_conquer_tree(make, n, nsub):
         assert root == ro and np.array_equal(par, po) and np.array_equal(lev, lo)
         g.set_state(0.0, r, v)
     g.close()
+
+
+@pytest.mark.parametrize("make", [half_lattice, lattice])
+@pytest.mark.parametrize("n", [512, 900, 3001, 8000])
+def test_step_tree_after_another_system(make, n):
+    """The step's tree of a tied system in a context whose scratch holds another system's sums."""
+    m, r, v = make(n)
+    _, r0, v0 = W.plummer(n, 43)
+    g = M.Integrator(m, r0, v0)
+    for _ in range(2):
+        g.set_state(0.0, r0, v0)
+        g.attempt(1e-6)
+        g.set_state(0.0, r, v)
+        root, par, lev, _ = g.mst(with_order=False)
+        ro, po, lo, _ = O.prim(g.state()["r"])
+        assert root == ro and np.array_equal(par, po) and np.array_equal(lev, lo)
+    g.close()
