@@ -34,9 +34,12 @@ struct FixWindow {
   float inv_max;  // 1 / r^2 limit: pairs closer than 2^-10 of the extent are not taken
 };
 
-// From the extents lo[3], hi[3] of the two tiles' bodies. The float copies of the positions err by
-// 2^-24 of the largest coordinate, which must not exceed 2^8 extents, so a float r^2 of a pair at the limit is within 12 % (the limit allows for 30 %).
-__device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi, bool ok) {
+// From the extents lo[3], hi[3] of the two tiles' bodies and, unless all masses are equal (which the
+// float bounds leave out), the exponent of the smallest mass (at least 2^em): every m / r^2 is at
+// least 2^(em - 2E - 2), and its float must not vanish or lose bits. The float copies of the
+// positions err by 2^-24 of the largest coordinate, which must not exceed 2^8 extents, so a float
+// r^2 of a pair at the limit is within 12 % (the limit allows for 30 %).
+__device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi, int em, bool eq, bool ok) {
   FixWindow w;
   const float ext = fmaxf(hi[0] - lo[0], fmaxf(hi[1] - lo[1], hi[2] - lo[2])) * (1.0f + 0x1p-18f);
   float big = 0.0f;
@@ -45,6 +48,7 @@ __device__ __forceinline__ FixWindow fix_window(const float* lo, const float* hi
   w.ok = ok && ext >= 0x1p-30f && big <= 256.0f * ext;
   const int E = (int)((__float_as_uint(ext) >> 23) & 255u) - 126;  // ext < 2^E
   w.u = E - 62;
+  w.ok &= eq || em - 2 * E > -118;
   const float r = ext * 0x1p-10f;
   w.inv_max = 1.0f / (1.3f * r * r);
   return w;
@@ -67,22 +71,24 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
     hi[c] = fmaxf(i_pad ? -kInf : __double2float_ru(pi3[c]), j_pad ? -kInf : __double2float_ru(pj3[c]));
     ok &= (i_pad || fabs(pi3[c]) < 0x1p50) && (j_pad || fabs(pj3[c]) < 0x1p50);  // false for NaN
   }
-  // masses within 2^-40 ... 2^40, so that the float bounds of m / r^2 neither overflow nor vanish
+  // masses within 2^-41 ... 2^40, so that the float bounds of m / r^2 do not overflow
   const int ei = mass_split(mi).e + 64, ej = mass_split(mj).e + 64;
   ok &= (i_pad || (ei > -40 && ei < 40)) && (j_pad || (ej > -40 && ej < 40));
+  const int em = min(i_pad ? 4096 : ei - 1, j_pad ? 4096 : ej - 1);
   bool eq = __all_sync(0xffffffffu, (i_pad || mi == m0) && (j_pad || mj == m0));
   ok = __all_sync(0xffffffffu, ok);
-  int key[6];
+  int key[7];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     key[c] = __reduce_min_sync(0xffffffffu, float_key(lo[c]));
     key[3 + c] = __reduce_max_sync(0xffffffffu, float_key(hi[c]));
   }
+  key[6] = __reduce_min_sync(0xffffffffu, em);
   if constexpr (NW > 1) {
     if (lane == 0) {
 #pragma unroll
-      for (int c = 0; c < 6; ++c) sbox[warp][c] = key[c];
-      sbox[warp][6] = (ok ? 1 : 0) | (eq ? 2 : 0);
+      for (int c = 0; c < 7; ++c) sbox[warp][c] = key[c];
+      sbox[warp][7] = (ok ? 1 : 0) | (eq ? 2 : 0);
     }
     __syncthreads();
 #pragma unroll
@@ -92,8 +98,9 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
         key[c] = min(key[c], sbox[w][c]);
         key[3 + c] = max(key[3 + c], sbox[w][3 + c]);
       }
-      ok &= (sbox[w][6] & 1) != 0;
-      eq &= (sbox[w][6] & 2) != 0;
+      key[6] = min(key[6], sbox[w][6]);
+      ok &= (sbox[w][7] & 1) != 0;
+      eq &= (sbox[w][7] & 2) != 0;
     }
   }
 #pragma unroll
@@ -101,7 +108,7 @@ __device__ __forceinline__ FixWindow tile_window(const double (&pi3)[3], const d
     lo[c] = key_float(key[c]);
     hi[c] = key_float(key[3 + c]);
   }
-  FixWindow fw = fix_window(lo, hi, ok);
+  FixWindow fw = fix_window(lo, hi, key[6], eq, ok);
   // The three components of a force share one unit. Where this warp's bodies lie flat (the mean
   // distance from the middle of the extent along one axis below an eighth of that along
   // another), the small component would keep fewer bits than binary64 sums do: not taken.
