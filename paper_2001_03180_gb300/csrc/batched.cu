@@ -331,8 +331,7 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
         sh.fx[lane] = fix_of(xj, fw.u);
         sh.fy[lane] = fix_of(yj, fw.u);
         sh.fz[lane] = fix_of(zj, fw.u);
-        sh.f[lane] = make_float4(__double2float_rn(xj), __double2float_rn(yj), __double2float_rn(zj),
-                                 __double2float_rn(mjb));
+        sh.f[lane] = make_float4(float_of(xj), float_of(yj), float_of(zj), sqrtf(float_of(mjb)));
         const MassSplit ms = fix_mass(mjb);
         sh.ms[lane] = ms.m;
         sh.me[lane] = ms.e;
@@ -350,7 +349,7 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
         __syncwarp();
         const SubTile t{sh.x,  sh.y,  sh.z,  sh.fx, sh.fy, sh.fz, sh.ms, sh.me, sh.f,
                         nullptr, sh.ax, sh.ay, sh.az, sh.bx, sh.by, sh.bz, sh.cj};
-        subtile_pairs<false>(body, t, fw, eq, m0, mw, k0, k1, lane);
+        subtile_pairs<false, 8>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] { return BodyPos{xi, yi, zi, 0.0}; });
         axi = body.ax;
         ayi = body.ay;
         azi = body.az;

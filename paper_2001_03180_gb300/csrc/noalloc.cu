@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(32 * W * W * S, 1)
   const double mi = i_pad ? 0.0 : m[i], mj = j_pad ? 0.0 : m[j], m0 = m[I * T];
   bool eq;
   FixWindow fw = tile_window<NW>(pi3, pj3, mi, mj, i_pad, j_pad, m0, sbox, &eq);
-  // masses that are not positive are legal here: FP64 throughout
-  fw.ok = __all_sync(0xffffffffu, fw.ok && (i_pad || mi > 0.0) && (j_pad || mj > 0.0));
+  // masses that are not positive are legal here: FP64 throughout (zero is outside the window's range)
+  fw.ok = __all_sync(0xffffffffu, fw.ok && (i_pad || __double2hiint(mi) >= 0) && (j_pad || __double2hiint(mj) >= 0));
   if (tid < T) {  // the warps of wi = 0, s = 0
     sx[tid] = pj3[0];
     sy[tid] = pj3[1];
@@ -115,8 +115,7 @@ __global__ void __launch_bounds__(32 * W * W * S, 1)
     sfx[tid] = fix_of(pj3[0], fw.u);
     sfy[tid] = fix_of(pj3[1], fw.u);
     sfz[tid] = fix_of(pj3[2], fw.u);
-    sf[tid] = make_float4(__double2float_rn(pj3[0]), __double2float_rn(pj3[1]), __double2float_rn(pj3[2]),
-                          __double2float_rn(mj));
+    sf[tid] = make_float4(float_of(pj3[0]), float_of(pj3[1]), float_of(pj3[2]), sqrtf(float_of(mj)));
     const MassSplit ms = fix_mass(mj);
     smm[tid] = ms.m;
     sme[tid] = ms.e;
@@ -135,7 +134,10 @@ __global__ void __launch_bounds__(32 * W * W * S, 1)
     const SubTile t{sx + js,       sy + js,       sz + js,       sfx + js,      sfy + js,      sfz + js,
                     smm + js,      sme + js,      sf + js,       sm + js,       sj3[warp][0],  sj3[warp][1],
                     sj3[warp][2],  sb,            sb + 32,       sb + 64,       scj[warp]};
-    subtile_pairs<true>(body, t, fw, eq, m0, mw, k0, k1, lane);
+    subtile_pairs<true, S < 4 ? 8 : 16 / S>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] {
+      return i_pad ? BodyPos{0.0, 0.0, 0.0, 0.0}
+                   : BodyPos{r[3 * (size_t)i], r[3 * (size_t)i + 1], r[3 * (size_t)i + 2], mi};
+    });
   }
   __syncwarp();
   si3[warp][0][lane] = body.ax;

@@ -252,8 +252,7 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
   sfx[tid] = fix_of(pj3[0], fw.u);
   sfy[tid] = fix_of(pj3[1], fw.u);
   sfz[tid] = fix_of(pj3[2], fw.u);
-  sf[tid] = make_float4(__double2float_rn(pj3[0]), __double2float_rn(pj3[1]), __double2float_rn(pj3[2]),
-                        __double2float_rn(mj));
+  sf[tid] = make_float4(float_of(pj3[0]), float_of(pj3[1]), float_of(pj3[2]), sqrtf(float_of(mj)));
   const MassSplit msj = fix_mass(mj);
   smm[tid] = msj.m;
   sme[tid] = msj.e;
@@ -277,7 +276,8 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
                                   n - j0 - js, self, lane);
     const SubTile t{sx + js,  sy + js,  sz + js,       sfx + js,      sfy + js,      sfz + js, smm + js, sme + js,
                     sf + js,  nullptr, &sax[warp][js], &say[warp][js], &saz[warp][js], sbx + wo,      sby + wo, sbz + wo, scj + wo};
-    subtile_pairs<false>(body, t, fw, eq, m0, mw, self ? 1 : 0, self ? 17 : 32, lane);
+    subtile_pairs<false, 8>(body, t, fw, eq, m0, mw, self ? 1 : 0, self ? 17 : 32, lane,
+                            [&] { return BodyPos{load_again(rx + i), load_again(ry + i), load_again(rz + i), 0.0}; });
   }
   __syncthreads();
   // the warps' partner sums, in warp order
@@ -387,8 +387,7 @@ k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __r
     sfx[lane] = fix_of(pj3[0], fw.u);
     sfy[lane] = fix_of(pj3[1], fw.u);
     sfz[lane] = fix_of(pj3[2], fw.u);
-    sf[lane] = make_float4(__double2float_rn(pj3[0]), __double2float_rn(pj3[1]), __double2float_rn(pj3[2]),
-                           __double2float_rn(mj));
+    sf[lane] = make_float4(float_of(pj3[0]), float_of(pj3[1]), float_of(pj3[2]), sqrtf(float_of(mj)));
     const MassSplit ms = fix_mass(mj);
     smm[lane] = ms.m;
     sme[lane] = ms.e;
@@ -424,7 +423,9 @@ k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __r
         near |= (n_d >= 2) & ((gpi == jq) | (sg[q] == i) | (pi == pj));
         mw |= near ? 1u << k : 0u;
       }
-    subtile_pairs<false>(body, t, fw, eq, m0, mw, k0, k1, lane);
+    subtile_pairs<false, S == 2 ? 8 : 16 / S>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] {
+      return BodyPos{load_again(rx + i), load_again(ry + i), load_again(rz + i), 0.0};
+    });
   }
   __syncwarp();
   si4[warp][0][lane] = body.ax;
