@@ -52,7 +52,8 @@ struct SysScalars {
   double t, B, H, M, U0, T0, eps, Ha;  // Ha: the fictitious step of the current attempt
   long long accepted, rejected, force_evals;
   int status;      // 0 running, 1 reached t_end, 2 time-iteration limit, -3 no convergence
-  int halvings, time_iters, go;  // go: the current attempt runs (1) or the system stopped (0)
+  int halvings, time_iters;
+  int go;          // the current attempt runs: 1, or 2 with its pair blocks swept; 0: the system stopped
 };
 
 // Per-body storage (doubles), offsets in units of n doubles (a 3-vector field spans 3).
@@ -283,11 +284,17 @@ struct WarpShared {
 // Pair loop of one system by one group: accelerations (3-vectors, times G) into a0 (the
 // group's first partial buffer; partial w at a0 + 3 n w) and the return value U. Ends with
 // the group synchronised and a0 complete.
+//
+// sweep: the 32 x 32 blocks are swept like a narrow last one, in FP64 separations and sums with the
+// integer pair scalars, without asking whether integers serve. The evaluation that starts an attempt
+// asks for every block (*left: the warp's blocks left to FP64 less those taken in integers), and where
+// most were left the attempt's others sweep: thin discs and systems with bodies far out took 4 to
+// 12 % longer in the blocks' own fallback (300 discs of 199 bodies 13.1 ms, 12.2 swept).
 template <int G>
 __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ m, const int* __restrict__ parent,
                           const int* __restrict__ gp, const int* __restrict__ coff, const int* __restrict__ cidx,
                           const double* r, const double* X, double* a0, WarpShared& sh, const GI& gi,
-                          double (*red)[kMaxG][3]) {
+                          double (*red)[kMaxG][3], bool sweep, int* left) {
   const int lane = gi.lane;
   double* a = a0 + (size_t)3 * n * gi.w;
   for (int v = lane; v < n; v += 32) {
@@ -323,7 +330,7 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
       // order), so that no two lanes update the same accumulator at a step.
       const int tail = n - J * 32;
       const int Wb = tail >= 32 ? 32 : (1 << (32 - __clz(tail - 1)));
-      if (Wb == 32) {  // the arithmetic of the large systems' pair loop
+      if (Wb == 32 && !sweep) {  // the arithmetic of the large systems' pair loop
         const double pi3[3] = {xi, yi, zi}, pj3[3] = {xj, yj, zj};
         const double m0 = m[I * 32];
         bool eq;
@@ -349,7 +356,9 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
         __syncwarp();
         const SubTile t{sh.x,  sh.y,  sh.z,  sh.fx, sh.fy, sh.fz, sh.ms, sh.me, sh.f,
                         nullptr, sh.ax, sh.ay, sh.az, sh.bx, sh.by, sh.bz, sh.cj};
-        subtile_pairs<false, 8>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] { return BodyPos{xi, yi, zi, 0.0}; });
+        const bool ints = subtile_pairs<false, 8>(body, t, fw, eq, m0, mw, k0, k1, lane,
+                                                  [&] { return BodyPos{xi, yi, zi, 0.0}; });
+        if (left) *left += ints ? -1 : 1;
         axi = body.ax;
         ayi = body.ay;
         azi = body.az;
@@ -566,7 +575,7 @@ __device__ __forceinline__ SysView sys_view(int s, const int* __restrict__ off, 
 // Start of an attempt, by a CTA of 128 G threads: the MST (Prim with exact FP64 keys) and
 // its children lists, the edge coordinates of the step start, the derivative information
 // (one force evaluation by group 0) and the step size. Leaves U0, T0, the attempt's H (Ha)
-// and go = 0 (system stops) or 1 in S; the caller synchronises before reading them.
+// and go = 0 (system stops), 1 or 2 in S; the caller synchronises before reading them.
 template <int G>
 __device__ void attempt_begin(const SysView& V, SysScalars* S, const BatchParams& P, double t_end, WarpShared* wsh,
                               unsigned long long* rk, int* ri, int* s_cnt, int* s_lev, double (*s_gred)[kMaxG][3]) {
@@ -695,7 +704,10 @@ __device__ void attempt_begin(const SysView& V, SysScalars* S, const BatchParams
   // ---- derivative information of the step start (group 0) and the step size
   if (gi.g == 0) {
     double* ga = V.F(B_GRP) + 12 * n;
-    const double U0 = gforces<G>(n, P.n_d, P.G, m, parent, gp, coff, cidx, R, X0, ga, wsh[warp], gi, s_gred);
+    int left = 0;
+    const double U0 =
+        gforces<G>(n, P.n_d, P.G, m, parent, gp, coff, cidx, R, X0, ga, wsh[warp], gi, s_gred, false, &left);
+    const bool sweep = gsum1<G>(lane == 0 ? (double)left : 0.0, gi, s_gred) > 0.0;
     double t2 = 0.0;
     for (int v = gi.t; v < n; v += 32 * G) {
       const double q0 = Vs[3 * v], q1 = Vs[3 * v + 1], q2 = Vs[3 * v + 2];
@@ -710,7 +722,7 @@ __device__ void attempt_begin(const SysView& V, SysScalars* S, const BatchParams
       S->U0 = U0;
       S->T0 = T0;
       S->Ha = Hs;
-      S->go = abort_ ? 0 : 1;
+      S->go = abort_ ? 0 : (sweep ? 2 : 1);
     }
   }
 }
@@ -731,6 +743,7 @@ __device__ void attempt_divisions(const SysView& V, const SysScalars* S, const B
   double* gv = gX + 9 * n;
   double* ga = gX + 12 * n;
   const double t0 = S->t, B = S->B, Mtot = S->M, T0 = S->T0, H = S->Ha, rM = 1.0 / Mtot;
+  const bool sweep = S->go == 2;
   int load[kGroups] = {0, 0, 0, 0};
   for (int k = K; k >= 1; --k) {
     int gsel = 0;
@@ -750,7 +763,8 @@ __device__ void attempt_divisions(const SysView& V, const SysScalars* S, const B
     gsync<G>(gi.g);
     grebuild<G>(n, m, parent, V.bylev, gX, gr, Mtot, rM, false, gi, s_gred);
     for (int tau = 1; tau <= nk; ++tau) {
-      const double U = gforces<G>(n, P.n_d, P.G, m, parent, V.gp, V.coff, V.cidx, gr, gX, ga, wsh, gi, s_gred);
+      const double U =
+          gforces<G>(n, P.n_d, P.G, m, parent, V.gp, V.coff, V.cidx, gr, gX, ga, wsh, gi, s_gred, sweep, nullptr);
       const double fk = delta / U;
       for (int v = gi.t; v < n; v += 32 * G) {
         const int p = parent[v];
@@ -1343,7 +1357,8 @@ k_batched_init(int nsys, const int* __restrict__ off, BatchParams P, const doubl
   // U with every pair Cartesian (Eq. 1), T
   int* ib = ibody + (size_t)o * 5;
   double* a = bd + (size_t)B_GRP * n + 12 * (size_t)n;
-  const double U = gforces<1>(n, 0, P.G, m, ib, ib + n, ib + 2 * n, ib + 3 * n + 1, R, R, a, wsh, gi, nullptr);
+  const double U = gforces<1>(n, 0, P.G, m, ib, ib + n, ib + 2 * n, ib + 3 * n + 1, R, R, a, wsh, gi, nullptr,
+                              false, nullptr);
   double t2 = 0.0;
   for (int v = lane; v < n; v += 32) {
     const double q0 = Vs[3 * v], q1 = Vs[3 * v + 1], q2 = Vs[3 * v + 2];

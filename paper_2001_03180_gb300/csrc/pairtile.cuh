@@ -232,9 +232,9 @@ __device__ __forceinline__ void bound_steps(const TilePos& b, const SubTile& t, 
 // (l + k) mod 32, unless bit k of its mask mw is set. m0: the common mass when eq. The fallback for
 // pairs that integers do not serve is the mixed FP64 / integer arithmetic, or (kPlain) FP64
 // throughout, which takes masses of any value and leaves NaN where bodies coincide; pos() reads
-// body i's binary64 position and mass for it.
+// body i's binary64 position and mass for it. True if integers served.
 template <bool kPlain, int kPre, typename Pos>
-__device__ __forceinline__ void subtile_pairs(TileBody& b, const SubTile& t, const FixWindow& fw, bool eq, double m0,
+__device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, const FixWindow& fw, bool eq, double m0,
                                               unsigned mw, int k0, int k1, int lane, Pos pos) {
   // The closest pair decides whether integers serve. It is looked at every kPre steps: where it
   // rules them out, it mostly does so at once (attempts at N = 10002 with 5 % of the bodies 10^3
@@ -260,7 +260,8 @@ __device__ __forceinline__ void subtile_pairs(TileBody& b, const SubTile& t, con
     }
     fj = __shfl_sync(0xffffffffu, fj, (lane - k1) & 31);  // held for partner lane + k1: to its own lane
   }
-  if (__all_sync(0xffffffffu, fw.ok && inv_hi <= fw.inv_max)) {
+  const bool ints = __all_sync(0xffffffffu, fw.ok && inv_hi <= fw.inv_max);
+  if (ints) {
     // accumulator units 2^L: forces and potentials below 2^58 units (the bounds hold within 1.5)
     const int Li = (int)(__float_as_uint(1.5f * fi) >> 23) - 184, Lj = (int)(__float_as_uint(1.5f * fj) >> 23) - 184,
               LU = (int)(__float_as_uint(1.5f * pu) >> 23) - 184;
@@ -361,6 +362,7 @@ __device__ __forceinline__ void subtile_pairs(TileBody& b, const SubTile& t, con
       __syncwarp();
     }
   }
+  return ints;
 }
 
 }  // namespace mstar
