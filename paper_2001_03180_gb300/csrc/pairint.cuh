@@ -24,6 +24,12 @@
 // body's accumulators is 2^-58 of a power of two at least 1.3 times the largest force of these 32
 // partners on that body, so a sum of up to 32 terms stays below 2^63 and a term is off by at most
 // a unit: a binary64 accumulation loses 2^-54 of the running sum per term.
+// Where all masses are equal the products are formed once, in the finer of the two bodies' units, and
+// shifted down for the other without rounding: half a unit per term too low on average there, at most
+// 2^-53 of the largest force of the 32 partners. Against long double sums (n = 64, 600, 2047 Plummer
+// spheres, in units of 2^-53 of a body's force) the mean error of a component is 0.00 to 0.08,
+// within its statistical error, and the rms error 0.4, 0.6 and 0.83; FP64 sums had 0.6, 0.8 and
+// 1.2, and rounded shifts 0.4, 0.6 and 0.65 for 9 % more time (N = 10002 attempts 32.0 against 29.5 ms).
 // The potential m_j / r is truncated to a unit of its own, 2^-58 of a power of two at least 1.3 and at
 // most 4 times the largest m_j / r among the body's partners that are not masked, whatever the body's
 // own mass and those of the other bodies: half a unit is given back for every term, so 32 terms err
