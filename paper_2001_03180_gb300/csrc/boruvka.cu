@@ -284,7 +284,9 @@ __device__ __forceinline__ void abs_bounds(double x, float& lo, float& hi) {
 // at N = 10002, in shared memory), the splitters are ranked by pointer doubling, and a second walk
 // gives every arc its rank. An arc that precedes its twin leads away from the root, and the
 // running sum of +1 (away) and -1 (back) along the tour is the level it reaches. Parent and level
-// do not depend on the order of the adjacency lists, which the atomic fill leaves open.
+// do not depend on the order of the adjacency lists, which the atomic fill leaves open. An edge list
+// that is no spanning tree gives the star around the root: whatever the list holds, every vertex gets
+// a parent and every walk up the tree ends.
 // 20 n bytes of shared memory hold the arcs as 16-bit numbers (2 (n - 1) < 2^16).
 // N = 601, 2050, 5003, 10002: 28, 57, 122 and 220 us before, 11, 18, 30 and 51 us now.
 constexpr int kNoSplitter = 0xffff;
@@ -303,7 +305,7 @@ k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, cons
   u16* pos = adj + 2 * n;                            // 2 n: place of each arc in adj; then its splitter; then the arc at each rank
   u16* succ = pos + 2 * n;                           // 2 n
   __shared__ unsigned long long rk[32];
-  __shared__ int ri[32], part[32], s_root;
+  __shared__ int ri[32], part[32], s_root, s_bare;
   __shared__ float s_hi;
   __shared__ int s_len[2][1024], s_nxt[2][1024];
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
@@ -326,7 +328,7 @@ k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, cons
     if (lane == 0) s_hi = __uint_as_float(u);
   }
   // (endpoints outside [0, n) cannot come from the tree builders; they are made 0 so that no
-  // shared-memory index leaves its array)
+  // shared-memory index leaves its array, and the list is then no tree)
   for (int e = tid; e < n - 1; e += nt) {
     int a = eu[e], b = ev[e];
     if ((unsigned)a >= (unsigned)n || (unsigned)b >= (unsigned)n) a = b = 0;
@@ -368,6 +370,7 @@ k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, cons
   }
   __syncthreads();
   if (tid == 0) {
+    s_bare = 0;
     for (int w = 1; w < nw; ++w)
       if (rk[w] < rk[0] || (rk[w] == rk[0] && ri[w] < ri[0])) {
         rk[0] = rk[w];
@@ -381,8 +384,13 @@ k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, cons
   const int b0 = min(n, tid * chunk), b1 = min(n, b0 + chunk);
   {
     int sum = 0, total;
-    for (int v = b0; v < b1; ++v) sum += off[v];
+    bool bare = false;
+    for (int v = b0; v < b1; ++v) {
+      sum += off[v];
+      bare |= off[v] == 0;
+    }
     sum = block_exclusive_scan(sum, part, &total);
+    if (bare) s_bare = 1;
     for (int v = b0; v < b1; ++v) {
       const int d = off[v];
       off[v] = sum;
@@ -390,13 +398,20 @@ k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, cons
     }
   }
   __syncthreads();
+  const int root = s_root;
+  auto star = [&] {
+    for (int v = tid; v < n; v += nt) {
+      parent[v] = v == root ? -1 : root;
+      level[v] = v != root;
+    }
+  };
+  if (s_bare) return star();  // a vertex without an edge
   for (int a = tid; a < na; a += nt) {
     const int p = atomicAdd(&off[src[a]], 1);
     adj[p] = (u16)a;
     pos[a] = (u16)p;
   }
   __syncthreads();
-  const int root = s_root;
   const int head = adj[root > 0 ? off[root - 1] : 0];
   for (int a = tid; a < na; a += nt) {  // the arc after a: the one after its twin around v
     const int t = a ^ 1, v = src[t], q = pos[t] + 1;
@@ -433,6 +448,7 @@ k_orient(int n, const double* __restrict__ X, const double* __restrict__ Y, cons
     s_nxt[h ^ 1][tid] = q ? s_nxt[h][q] : 0;
     __syncthreads();
   }
+  if (s_len[h][0] != na) return star();  // not connected
   if (mine >= 0) {
     int k = na - s_len[h][tid], a = mine;  // rank of the splitter
     for (int j = 0; j < len; ++j, ++k) {

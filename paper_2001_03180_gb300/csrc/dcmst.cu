@@ -470,7 +470,8 @@ k_dc_local_prim(const int* __restrict__ ncell, const int* __restrict__ leaf_star
     for (int w = 0; w < kLpThreads / 32; ++w)
       if (lp_less(red[it & 1][w], best)) best = red[it & 1][w];
     if ((best.q % kLpThreads) == tid) {
-      eu[e0 + it - 1] = kp[best.q];
+      // (no parent: every distance to the body overflows or is NaN; any edge keeps the tree whole)
+      eu[e0 + it - 1] = kp[best.q] >= 0 ? kp[best.q] : st.v;
       ev[e0 + it - 1] = best.v;
       kp[best.q] = -2;
     }
