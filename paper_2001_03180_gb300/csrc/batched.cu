@@ -285,11 +285,16 @@ struct WarpShared {
 // group's first partial buffer; partial w at a0 + 3 n w) and the return value U. Ends with
 // the group synchronised and a0 complete.
 //
-// sweep: the 32 x 32 blocks are swept like a narrow last one, in FP64 separations and sums with the
-// integer pair scalars, without asking whether integers serve. The evaluation that starts an attempt
-// asks for every block (*left: the warp's blocks left to FP64 less those taken in integers), and where
-// most were left the attempt's others sweep: thin discs and systems with bodies far out took 4 to
-// 12 % longer in the blocks' own fallback (300 discs of 199 bodies 13.1 ms, 12.2 swept).
+// A 32 x 32 block that integers do not serve is swept like a narrow last one, in FP64 separations and
+// sums with the integer pair scalars. sweep: all are, without asking. The evaluation that starts an
+// attempt asks for every block (*left: the warp's blocks left to FP64 less those taken in integers),
+// and where most were left the attempt's others sweep: thin discs and systems with bodies far out
+// took 4 to 12 % longer otherwise (300 discs of 199 bodies 13.1 ms, 12.2 swept).
+//
+// The loops are kept short (no unrolling): kernels of several widths share an SM in a mixed batch, and
+// its instruction cache. With the loops unrolled as in the large systems' kernels and the mixed
+// fallback beside the sweep, 330 KB of code a kernel instead of 280, 4096 mixed systems took 14.0 ms
+// a launch, 11.6 now; batches of one width take the same time within 2 %.
 template <int G>
 __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ m, const int* __restrict__ parent,
                           const int* __restrict__ gp, const int* __restrict__ coff, const int* __restrict__ cidx,
@@ -330,7 +335,8 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
       // order), so that no two lanes update the same accumulator at a step.
       const int tail = n - J * 32;
       const int Wb = tail >= 32 ? 32 : (1 << (32 - __clz(tail - 1)));
-      if (Wb == 32 && !sweep) {  // the arithmetic of the large systems' pair loop
+      bool ints = false;
+      if (Wb == 32 && !sweep) {  // the integers of the large systems' pair loop
         const double pi3[3] = {xi, yi, zi}, pj3[3] = {xj, yj, zj};
         const double m0 = m[I * 32];
         bool eq;
@@ -345,6 +351,7 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
         const int k0 = self ? 1 : 0, k1 = self ? 17 : 32;
         unsigned mw = mask_word(nullptr, ipad, tail, self, lane);
         if (nd1)
+#pragma unroll 1
           for (int k = k0; k < k1; ++k) {
             const int q = (lane + k) & 31, j = J * 32 + q;
             const int pj = __shfl_sync(0xffffffffu, pjb, q), gj = __shfl_sync(0xffffffffu, gjb, q);
@@ -356,14 +363,14 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
         __syncwarp();
         const SubTile t{sh.x,  sh.y,  sh.z,  sh.fx, sh.fy, sh.fz, sh.ms, sh.me, sh.f,
                         nullptr, sh.ax, sh.ay, sh.az, sh.bx, sh.by, sh.bz, sh.cj};
-        const bool ints = subtile_pairs<false, 8>(body, t, fw, eq, m0, mw, k0, k1, lane,
-                                                  [&] { return BodyPos{xi, yi, zi, 0.0}; });
+        ints = subtile_pairs<Fallback::none, 4, 1>(body, t, fw, eq, m0, mw, k0, k1, lane, [] { return BodyPos{}; });
         if (left) *left += ints ? -1 : 1;
         axi = body.ax;
         ayi = body.ay;
         azi = body.az;
         ui = body.u_sum();
-      } else {
+      }
+      if (!ints) {
         const MassSplit msi = mass_split(ipad ? 1.0 : mi);
         const MassSplit ms = mass_split(jpad ? 1.0 : mjb);
         sh.mm[lane] = mjb;
@@ -374,6 +381,7 @@ __device__ double gforces(int n, int n_d, double Gc, const double* __restrict__ 
         __syncwarp();
         const int cb = lane & ~(Wb - 1);
         const int kbeg = self ? 1 : 0, kend = self ? Wb / 2 + 1 : Wb;
+#pragma unroll 1
         for (int k = kbeg; k < kend; ++k) {
           const int jl = (lane + k) & (Wb - 1);
           const int ja = cb + jl;
@@ -883,10 +891,13 @@ template <int G>
 __global__ void __launch_bounds__(128 * G) k_batched_step(MSTAR_BSTEP_ARGS) {
   extern __shared__ __align__(16) unsigned char wsh_mem[];  // 4 G WarpShared
   WarpShared* wsh = reinterpret_cast<WarpShared*>(wsh_mem);
+  // the tree's lists are built where the pair loop's blocks come later: four G = 1 and two G = 2 CTAs,
+  // as many as the registers allow, then fit 64 KB (apply_schedule)
+  int* s_cnt = reinterpret_cast<int*>(wsh_mem);  // kBMaxN + 1
+  int* s_lev = s_cnt + kBMaxN + 1;               // kBMaxN
+  static_assert((2 * kBMaxN + 1) * sizeof(int) <= 4 * G * sizeof(WarpShared), "the lists must fit");
   __shared__ unsigned long long rk[4 * G];
   __shared__ int ri[4 * G];
-  __shared__ int s_cnt[kBMaxN + 1];
-  __shared__ int s_lev[kBMaxN];
   __shared__ double s_red[4 * G];
   __shared__ double s_gred[kGroups][kMaxG][3];
   __shared__ int s_flag;
@@ -913,10 +924,13 @@ template <int G>
 __global__ void __launch_bounds__(128 * G) k_bsplit_begin(MSTAR_BSTEP_ARGS) {
   extern __shared__ __align__(16) unsigned char wsh_mem[];  // 4 G WarpShared
   WarpShared* wsh = reinterpret_cast<WarpShared*>(wsh_mem);
+  // the tree's lists are built where the pair loop's blocks come later: four G = 1 and two G = 2 CTAs,
+  // as many as the registers allow, then fit 64 KB (apply_schedule)
+  int* s_cnt = reinterpret_cast<int*>(wsh_mem);  // kBMaxN + 1
+  int* s_lev = s_cnt + kBMaxN + 1;               // kBMaxN
+  static_assert((2 * kBMaxN + 1) * sizeof(int) <= 4 * G * sizeof(WarpShared), "the lists must fit");
   __shared__ unsigned long long rk[4 * G];
   __shared__ int ri[4 * G];
-  __shared__ int s_cnt[kBMaxN + 1];
-  __shared__ int s_lev[kBMaxN];
   __shared__ double s_gred[kGroups][kMaxG][3];
   if ((int)blockIdx.x >= count) return;
   const int s = order[blockIdx.x];
@@ -1542,6 +1556,11 @@ int apply_schedule(mstar_batch* b, const int* sched) {
                       int prio, cudaGraphNode_t* node) {
     if (smem && cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return false;
+    // One split of the on-chip memory for every node, so that CTAs of different nodes can share an SM:
+    // 64 KB of shared memory, the rest L1 for the systems' state. Left to the driver each kernel gets
+    // its own split, and the nodes run one after another (4096 mixed systems: 14.3 ms a launch against
+    // 12.0; 32, 100, 132, 196 and 228 KB: 17.7, 14.2, 14.5, 14.9 and 15.1). A hint; failure is harmless.
+    cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
     cudaKernelNodeParams kp{};
     kp.func = func;
     kp.gridDim = grid;

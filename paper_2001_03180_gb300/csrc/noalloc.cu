@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(32 * W * W * S, 1)
     const SubTile t{sx + js,       sy + js,       sz + js,       sfx + js,      sfy + js,      sfz + js,
                     smm + js,      sme + js,      sf + js,       sm + js,       sj3[warp][0],  sj3[warp][1],
                     sj3[warp][2],  sb,            sb + 32,       sb + 64,       scj[warp]};
-    subtile_pairs<true, S < 4 ? 8 : 16 / S>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] {
+    subtile_pairs<Fallback::plain, S < 4 ? 8 : 16 / S, 2>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] {
       return i_pad ? BodyPos{0.0, 0.0, 0.0, 0.0}
                    : BodyPos{r[3 * (size_t)i], r[3 * (size_t)i + 1], r[3 * (size_t)i + 2], mi};
     });

@@ -276,8 +276,8 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
                                   n - j0 - js, self, lane);
     const SubTile t{sx + js,  sy + js,  sz + js,       sfx + js,      sfy + js,      sfz + js, smm + js, sme + js,
                     sf + js,  nullptr, &sax[warp][js], &say[warp][js], &saz[warp][js], sbx + wo,      sby + wo, sbz + wo, scj + wo};
-    subtile_pairs<false, 8>(body, t, fw, eq, m0, mw, self ? 1 : 0, self ? 17 : 32, lane,
-                            [&] { return BodyPos{load_again(rx + i), load_again(ry + i), load_again(rz + i), 0.0}; });
+    subtile_pairs<Fallback::mixed, 8, 2>(body, t, fw, eq, m0, mw, self ? 1 : 0, self ? 17 : 32, lane,
+                                         [&] { return BodyPos{load_again(rx + i), load_again(ry + i), load_again(rz + i), 0.0}; });
   }
   __syncthreads();
   // the warps' partner sums, in warp order
@@ -423,7 +423,7 @@ k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __r
         near |= (n_d >= 2) & ((gpi == jq) | (sg[q] == i) | (pi == pj));
         mw |= near ? 1u << k : 0u;
       }
-    subtile_pairs<false, S == 2 ? 8 : 16 / S>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] {
+    subtile_pairs<Fallback::mixed, S == 2 ? 8 : 16 / S, 2>(body, t, fw, eq, m0, mw, k0, k1, lane, [&] {
       return BodyPos{load_again(rx + i), load_again(ry + i), load_again(rz + i), 0.0};
     });
   }

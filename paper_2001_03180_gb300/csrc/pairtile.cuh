@@ -230,10 +230,12 @@ __device__ __forceinline__ void bound_steps(const TilePos& b, const SubTile& t, 
 
 // Steps [k0, k1) of the warp's rotation (a multiple of kPre of them): at step k lane l meets partner
 // (l + k) mod 32, unless bit k of its mask mw is set. m0: the common mass when eq. The fallback for
-// pairs that integers do not serve is the mixed FP64 / integer arithmetic, or (kPlain) FP64
-// throughout, which takes masses of any value and leaves NaN where bodies coincide; pos() reads
-// body i's binary64 position and mass for it. True if integers served.
-template <bool kPlain, int kPre, typename Pos>
+// pairs that integers do not serve is the mixed FP64 / integer arithmetic, FP64 throughout, which
+// takes masses of any value and leaves NaN where bodies coincide, or the caller's; pos() reads body
+// i's binary64 position and mass for it. True if integers served. kUnroll: steps of the integer
+// loops in a row, for kernels that have the SM to themselves two.
+enum class Fallback { mixed, plain, none };
+template <Fallback kFallback, int kPre, int kUnroll, typename Pos>
 __device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, const FixWindow& fw, bool eq, double m0,
                                               unsigned mw, int k0, int k1, int lane, Pos pos) {
   // The closest pair decides whether integers serve. It is looked at every kPre steps: where it
@@ -276,7 +278,7 @@ __device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, con
     unsigned long long ui = __popc(~mw & (0xffffffffu >> (32 - k1) & 0xffffffffu << k0)) / 2;
     double si = exp2_int(Li), sj = exp2_int(Lj), su = exp2_int(LU);
     if (eq) {
-#pragma unroll 2
+#pragma unroll kUnroll
       for (int k = k0; k < k1; ++k) {
         const int r = (lane + k) & 31;
         FixAcc aj{t.bx[r], t.by[r], t.bz[r]};
@@ -290,7 +292,7 @@ __device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, con
       sj *= m0;
       su *= m0;
     } else {
-#pragma unroll 2
+#pragma unroll kUnroll
       for (int k = k0; k < k1; ++k) {
         const int r = (lane + k) & 31;
         FixAcc aj{t.bx[r], t.by[r], t.bz[r]};
@@ -311,7 +313,7 @@ __device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, con
     t.jy[lane] = fma((double)(t.by[lane] - bias), sj, t.jy[lane]);
     t.jz[lane] = fma((double)(t.bz[lane] - bias), sj, t.jz[lane]);
     __syncwarp();
-  } else if constexpr (kPlain) {
+  } else if constexpr (kFallback == Fallback::plain) {
     const BodyPos bi = pos();
 #pragma unroll 1
     for (int k = k0; k < k1; ++k) {
@@ -330,7 +332,7 @@ __device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, con
       t.jz[r] = fma(si, dz, t.jz[r]);
       __syncwarp();
     }
-  } else {
+  } else if constexpr (kFallback == Fallback::mixed) {
     const BodyPos bi = pos();
 #pragma unroll 2
     for (int k = k0; k < k1; ++k) {
