@@ -17,7 +17,13 @@
  * time (Sec. 2.4).
  *
  * Conventions for every entry point:
- *  - All arithmetic is IEEE binary64 (FP64). G defaults to 1.
+ *  - Inputs, state and results are IEEE binary64 (FP64), and so is the arithmetic but for the
+ *    pair sums. There the interaction of two bodies runs in 64-bit fixed point with units that
+ *    follow the positions, masses and forces (float estimates choose the units, no result): a
+ *    term errs by a few 2^-53 of itself and a sum by no more than one accumulated in binary64,
+ *    relative to the sum of its terms' magnitudes, for any ratio of the masses. Bodies whose
+ *    lengths or masses do not fit such units take binary64 separations and sums.
+ *    G defaults to 1.
  *  - Arrays of vectors are n x 3 row-major doubles (x0 y0 z0 x1 ...).
  *  - Array arguments may be host or device pointers; the library detects which with
  *    cudaPointerGetAttributes. The caller owns every array it passes; inputs are copied,
@@ -88,7 +94,8 @@ typedef struct {
   int division_schedule; /* how an attempt's k_fix divisions are issued: 1 level by level (the
                         kernels of a substep level for every division active at it: one CTA per
                         division for up to 160 padded bodies, a thread-block cluster per division
-                        for up to 576, else one launch per kernel; all bit-identical), 2 each
+                        for up to 576, else one launch per kernel; the cluster's results are
+                        those of the separate launches, bit for bit), 2 each
                         division on its own stream (longer divisions at higher priority), so that
                         one division's small kernels overlap another's pair loop, 3 each division
                         on one CTA, or a cluster of them (division_cluster), from its first drift
@@ -120,7 +127,10 @@ typedef struct {
 
 MSTAR_API void mstar_default_params(mstar_params* p);
 
-/* Device bytes a context for n bodies needs under p (for a caller-provided workspace). */
+/* Device bytes a context for n bodies needs under p (for a caller-provided workspace). Mostly the
+   pair loop's partial sums, 32 (k_fix + 1) n^2 / pair_tile bytes (600 MB at n = 8192 with the
+   default parameters), and with pair_split 1 the near-pair words, n^2 / 8 bytes. The figure belongs to
+   this version of the library: ask for it rather than keep one. */
 MSTAR_API size_t mstar_workspace_bytes(int n, const mstar_params* p);
 
 /* Create a context: copies m[n] (> 0), r[n x 3], v[n x 3], shifts them to the centre-of-

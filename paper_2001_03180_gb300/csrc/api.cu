@@ -544,11 +544,11 @@ int vectors_out(mstar_ctx* c, const double* planes, double* dst) {
 }
 
 // Pair tile of 32 W bodies by system size, from a sweep of full GBS steps on Plummer spheres. One
-// warp per CTA waits for no other: W = 1, 2, 4 take 5.26, 5.43, 5.43 ms at N = 4096, 7.75, 8.23, 8.47
-// at 5003, 18.8, 19.6, 19.3 at 8000 and 29.5, 30.8, 30.0 at 10002. Above 8192 the 128-body tiles
+// warp per CTA waits for no other: W = 1, 2, 4 take 5.23, 5.30, 5.24 ms at N = 4096, 7.76, 7.99, 8.24
+// at 5003, 19.0, 19.4, 19.1 at 8000 and 29.5, 30.4, 29.8 at 10002. Above 8192 the 128-body tiles
 // keep the partial sums (slots x tiles x 4 x npad doubles, 604 MB at N = 8192 with 32-body tiles) a
 // quarter as large for 2 % of the speed. Up to 768 bodies a tile pair's steps are split over four
-// warps (pair_split 4; 0.91 against 0.93 ms at N = 601, equal at 800, 3 % slower at 900).
+// warps (pair_split 4; 0.81 against 0.86 ms at N = 601, 0.93 against 0.94 at 768, 2 % slower at 900).
 int choose_tile_warps(int n) { return n <= 8192 ? 1 : 4; }
 
 size_t workspace_bytes(int n, const mstar_params& p, int* npad_out, int* W_out) {

@@ -74,10 +74,10 @@ __device__ __forceinline__ void na_tile_pair(int tp, int NT, int& I, int& J) {
 
 // Symmetric tiled pair loop over Cartesian separations (every pair far) in the arithmetic of
 // pairtile.cuh: one CTA per pair of tiles of 32 W bodies, one warp per pair of 32-body sub-tiles and
-// range of 32 / S rotation steps. Bound by the integer pipe above n = 1024 (22 us of 39 at n = 2047),
+// range of 32 / S rotation steps. Bound by the integer pipe above n = 1024 (22 us of 42 at n = 2047),
 // by latency below: prologue, one short chain of steps, the sums, two launches. The FP64 loop over
-// four-warp CTAs this replaced took 116 us at n = 100, 135 at 1024 and 137 at 2047 for four launches;
-// now 14.6, 22.7 and 39.2.
+// four-warp CTAs this replaced took 103 us at n = 100, 127 at 1024 and 130 at 2047 for four launches
+// (calls back to back on the stream); now 8.8, 17.0 and 42.5.
 template <int W, int S>
 __global__ void __launch_bounds__(32 * W * W * S, 1)
     k_na_tiles(int n, int npad, int NT, const double* __restrict__ m, const double* __restrict__ r,

@@ -10,19 +10,21 @@
 //  - integer (pairint.cuh): the whole interaction on the integer and FP32 pipes, accumulated in
 //    64-bit fixed point over the sub-tile and added to the FP64 sums once per sub-tile. The FP64
 //    pipe bound the mixed loop (9 instructions of 16 cycles per SM per warp step, 165 cycles
-//    measured); this one is bound by the integer multiply-adds (fmaheavy 76 % busy) at about 80,
-//    70 where all masses of the tile pair are equal. One force evaluation at N = 10002: 0.87 ->
-//    0.42 ms inside an attempt; attempts 61.3 -> 30.5 ms, at N = 2050 3.24 -> 2.11 ms.
+//    measured); this one is bound by the integer multiply-adds, 78 cycles a warp step in a loop of
+//    its own, 65 where all masses of the tile pair are equal. Attempts at N = 10002 61.1 -> 29.6 ms
+//    (one force evaluation in them 0.84 -> 0.41 ms), at N = 2050 3.22 -> 1.88 ms.
 //  - mixed, for the sub-tile pairs the integer window does not cover: a flat or very wide tile
 //    pair, masses or coordinates outside its exponent range, or an unmasked pair closer than
 //    2^-10 of the tile pair's extent (about 1 % of random sub-tile pairs of a Plummer sphere).
 //    There the FP64 pipe issues the separation (3 DADD) and the two force accumulations (6
 //    DFMA); r^2, 1/r, 1/r^3 and the mass products run on the integer pipe (pair_scalars_core), and
 //    so does the force-function sum: m_j / r is a 64-bit product of significands added exactly
-//    into a 128-bit fixed-point accumulator (UAcc).
-// A float pass over the sub-tile's pairs (17 instructions a pair) finds the closest pair, which
-// decides, and bounds of the largest force on each body, which set its accumulators' units. Both
-// are functions of the positions and masses alone, so results do not depend on timing.
+//    into a 128-bit fixed-point accumulator (UAcc). A system that is taken here throughout (a thin
+//    disc, or 5 % of the bodies 10^3 core radii out) gains nothing: attempts 62.1 -> 63.6 ms at
+//    N = 10002, 16.2 -> 16.8 at 5003, against the loop that knew only this arithmetic.
+// A float pass over the sub-tile's pairs finds the closest pair, which decides, and bounds of the
+// largest force on each body and the largest m_j / r, which set its accumulators' units. All are
+// functions of the positions and masses alone, so results do not depend on timing.
 //
 // Tiles: the N bodies form NT tiles of T = 32*W. CTA (I, J), I <= J, owns the I-tile as
 // "i" bodies (one per thread, accumulators in registers) and stages the J-tile ("j"
@@ -206,8 +208,9 @@ __device__ __forceinline__ void near_block(int n, int npad, int slot, int n_d, c
   }
 }
 
-// 24 warps per SM (80 registers, 100 bytes spilt outside the pair loops): attempts at N = 10002
-// took 31.5, 31.3, 30.5 and 30.4 ms with 16, 20, 24 and 28.
+// 24 warps per SM (80 registers; with W > 1 some 100 bytes spilt outside the pair loops). With 16, 20,
+// 24 and 28, attempts at N = 10002 (W = 4) took 30.8, 29.6, 29.8 and 29.2 ms, at N = 5003 (W = 1)
+// 8.40, 7.89, 7.75 and 7.80.
 template <int W>
 __global__ void __launch_bounds__(32 * W, 24 / W)
 k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __restrict__ m,
@@ -339,9 +342,9 @@ k_pair_tiles(int n, int npad, int NT, int slot_lo, int n_d, const double* __rest
 // [32 w / S, 32 (w + 1) / S) of an off-diagonal pair and [1 + 16 w / S, 1 + 16 (w + 1) / S) of a
 // diagonal one, keeping its own i-side and partner sums; the S copies are added in warp order at the
 // end. At N ~ 10^2 to 10^3 a tile pair's 32 dependent steps in one warp bind the launch; S warps
-// shorten them S-fold. What does not shrink is done once, by warp 0 (conversions and window: some
-// 500 cycles of FP64 pipe), or binds larger S (a warp's flush to FP64: 14 FP64 instructions).
-// Attempts with S = 1, 2, 4, 8: 0.83, 0.77, 0.73, 0.73 ms at N = 256, 0.80, 0.76, 0.73, 0.80 at 512.
+// shorten them S-fold. What does not shrink is done once, by warp 0 (conversions and window), or
+// binds larger S (a warp's flush to FP64: 14 FP64 instructions). Attempts with S = 1, 2, 4, 8:
+// 0.67, 0.58, 0.54, 0.56 ms at N = 256, 0.78, 0.71, 0.68, 0.74 at 512.
 template <int S>
 __global__ void __launch_bounds__(32 * S, 24 / S)
 k_pair_tiles_ks(int n, int npad, int NT, int slot_lo, int n_d, const double* __restrict__ m,

@@ -26,7 +26,7 @@
 // a unit: a binary64 accumulation loses 2^-54 of the running sum per term.
 // Where all masses are equal the products are formed once, in the finer of the two bodies' units, and
 // shifted down for the other without rounding: half a unit per term too low on average there, at most
-// 2^-53 of the largest force of the 32 partners. Against long double sums (n = 64, 600, 2047 Plummer
+// 2^-52 of the largest force of the 32 partners in all. Against long double sums (n = 64, 600, 2047 Plummer
 // spheres, in units of 2^-53 of a body's force) the mean error of a component is 0.00 to 0.08,
 // within its statistical error, and the rms error 0.4, 0.6 and 0.83; FP64 sums had 0.6, 0.8 and
 // 1.2, and rounded shifts 0.4, 0.6 and 0.65 for 9 % more time (N = 10002 attempts 32.0 against 29.5 ms).

@@ -233,7 +233,7 @@ __device__ __forceinline__ void bound_steps(const TilePos& b, const SubTile& t, 
 // pairs that integers do not serve is the mixed FP64 / integer arithmetic, FP64 throughout, which
 // takes masses of any value and leaves NaN where bodies coincide, or the caller's; pos() reads body
 // i's binary64 position and mass for it. True if integers served. kUnroll: steps of the integer
-// loops in a row, for kernels that have the SM to themselves two.
+// loops written out in a row (two where code size does not count).
 enum class Fallback { mixed, plain, none };
 template <Fallback kFallback, int kPre, int kUnroll, typename Pos>
 __device__ __forceinline__ bool subtile_pairs(TileBody& b, const SubTile& t, const FixWindow& fw, bool eq, double m0,
