@@ -45,17 +45,22 @@ NOMINAL_FP64_TFLOPS = 1.25
 DFMA_PER_CLK_PER_SM = 2
 NUM_SMS = 152
 L2_FLUSH_BYTES = 256 << 20
-# Figures from ncu captures of k_pair_tiles<4> (128-body tiles) at N = 10002, valid for the kernel
+# Figures from ncu captures of k_pair_tiles at N = 10002 by tile (bodies), valid for the kernel
 # built from the sources whose SHA-256 (PAIR_SOURCES in order) starts with the given prefix; for
-# other sources or another tile the bench reports them as null.
+# other sources or another tiling the bench reports them as null.
 #  - DRAM bytes (read + write) of one launch by the number of division slots it evaluates;
 #    an attempt launches the kernel for 1 (step start), 8, 8, 7, 7, ..., 1, 1 slots;
 #  - active fractions of the pipe that takes the 32 x 32-bit products (FMA heavy) and of the FP64 pipe.
 PAIR_SOURCES = ("pair.cu", "pairtile.cuh", "pairint.cuh", "device.cuh")
-PAIR_TILE_SRC_SHA = "5467a1591a52becb"
-PAIR_TILE_DRAM_BYTES_BY_SLOTS = {}  # not captured for these sources
-PAIR_TILE_FMAHEAVY_PIPE_NCU = 0.561
-PAIR_TILE_FP64_PIPE_NCU = 0.302
+PAIR_TILE_SRC_SHA = "dd543aaf4406461b"
+PAIR_TILE_NCU = {
+    128: {"fma_heavy": 0.563, "fp64": 0.122,
+          "dram_by_slots": {1: 3.53e6, 2: 7.76e6, 3: 9.62e6, 4: 11.49e6, 5: 13.42e6, 6: 15.74e6, 7: 18.16e6,
+                            8: 24.47e6}},
+    32: {"fma_heavy": 0.577, "fp64": 0.136,
+         "dram_by_slots": {1: 49.1e6, 2: 152.6e6, 3: 163.5e6, 4: 172.3e6, 5: 181.4e6, 6: 190.3e6, 7: 198.4e6,
+                           8: 210.8e6}},
+}
 ATTEMPT_SLOT_PATTERN = [1] + [k for k in range(8, 0, -1) for _ in range(2)]
 # Algorithmic DRAM bytes of one force evaluation per body: positions 24 and mass 8 read,
 # accelerations 24 written (parent and grandparent indices are another 8 read).
@@ -669,11 +674,11 @@ def run_mstar(args):
     achieved = FLOPS_PER_UNORDERED_PAIR * pairs_per_launch / (avg_ms * 1e-3) / 1e12
     clk_mhz = clocks_prof.get("sm_mhz") or 2070.0
     fp64_peak = 2.0 * DFMA_PER_CLK_PER_SM * NUM_SMS * clk_mhz * 1e6 / 1e12
-    sha_ok = pair_source_sha() == PAIR_TILE_SRC_SHA and (tile, split) == (128, 1)
+    ncu = PAIR_TILE_NCU.get(tile) if split == 1 and pair_source_sha() == PAIR_TILE_SRC_SHA else None
     slots_per_launch = prof.force_evals / max(prof.pair_launches, 1)
     # per launch, averaged over an attempt's launches (the pattern of slot counts is fixed)
-    traffic = (sum(PAIR_TILE_DRAM_BYTES_BY_SLOTS[k] for k in ATTEMPT_SLOT_PATTERN) / len(ATTEMPT_SLOT_PATTERN)
-               if sha_ok and PAIR_TILE_DRAM_BYTES_BY_SLOTS else None)
+    traffic = (sum(ncu["dram_by_slots"][k] for k in ATTEMPT_SLOT_PATTERN) / len(ATTEMPT_SLOT_PATTERN)
+               if ncu else None)
     algo_bytes = ALGO_BYTES_PER_BODY_EVAL * n * slots_per_launch
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp64_peak, "traffic": traffic,
@@ -689,11 +694,11 @@ def run_mstar(args):
                 "frac_above_1_because": ("the pairs run in 64-bit fixed point on the integer pipe: separations, r^2, "
                                          "1/r, r^-3, mass scalings and accumulations without FP64 instructions; the "
                                          "FP64 peak is the algorithm's yardstick, not what binds the kernel"),
-                "fma_heavy_pipe_util_ncu": PAIR_TILE_FMAHEAVY_PIPE_NCU if sha_ok else None,
-                "fp64_pipe_util_ncu": PAIR_TILE_FP64_PIPE_NCU if sha_ok else None,
+                "fma_heavy_pipe_util_ncu": ncu["fma_heavy"] if ncu else None,
+                "fp64_pipe_util_ncu": ncu["fp64"] if ncu else None,
                 "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum per launch by slot count, "
                                    "averaged over an attempt's 17 launches; null when the kernel's sources "
-                                   "differ from the captured ones" + ("" if sha_ok else " (they differ)")),
+                                   "or its tiling differ from the captured ones" + ("" if ncu else " (they differ)")),
                 "algorithmic_bytes": algo_bytes,
                 "traffic_over_algorithmic": traffic / algo_bytes if traffic else None,
                 "survey_unit_tflops": FLOPS_PER_ORDERED_PAIR_NONSYM * 2 * pairs_per_launch / (avg_ms * 1e-3) / 1e12,
@@ -748,6 +753,8 @@ def run_mstar(args):
                "config": {"workload": WORKLOAD_DESC, "n": n, "gbs_steps_per_bench_step": 1,
                           "l2": "flushed between steps (256 MiB write)",
                           "parallelism": "replicas" if world > 1 else "single",
+                          "arithmetic": "binary64 state, edge vectors and sums over tiles; pairs in 64-bit fixed point "
+                                        "or in binary64",
                           "division_schedule": ("one CTA per division" if len(m) <= 96 else
                                           ("a stream per division" if len(m) >= 1000 else "level by level")),
                     "pair_tile": tile, "pair_split": split, "pair_tile_tuner_ms_per_attempt": tile_ms},
